@@ -875,6 +875,7 @@ static pfmbem_status build_plan(pfmbem* h, const int* npf, const double* nodes) 
     h->hfib_geo[3 * i + 1] = sy;
     h->hfib_geo[3 * i + 2] = sr / n;
   }
+  h->hmax = hmax;
   if (h->opt.tree == 1) return build_plan_tri(h, nodes, foff, c, t, nu, len, fib, hmax, t0);
   if (h->opt.tree != 0) return fail(h, PFMBEM_EINVAL, "tree must be 0 (square) or 1 (triangle)");
   if (0.5 * k * hmax > 4.0) return fail(h, PFMBEM_EINVAL, "elements longer than 8/k");
@@ -2700,7 +2701,8 @@ pfmbem_status pfmbem_self_terms(pfmbem_t h, double* out) {
 namespace {
 // Scattered field and/or its x1-derivative at host or device points (shared by
 // pfmbem_field, pfmbem_field_dx1 and pfmbem_etc).
-pfmbem_status field_points(pfmbem* h, const double* psi, int npts, const double* pts, double* u, double* du) {
+pfmbem_status field_points(pfmbem* h, const double* psi, int npts, const double* pts, double* u, double* du,
+                           bool by_tree = false) {
   const size_t n = 2 * (size_t)h->E;
   // host copy of the points for the validity check
   std::vector<double> hp(2 * (size_t)npts);
@@ -2725,7 +2727,7 @@ pfmbem_status field_points(pfmbem* h, const double* psi, int npts, const double*
   if (!pd || !ud) return fail(h, PFMBEM_ENOMEM, "field buffers");
   CK(cudaMemcpyAsync(pd, hp.data(), sizeof(double2) * npts, cudaMemcpyHostToDevice, h->stream));
   CK(k_field_prepare(h, psid));
-  CK(k_field(h, psid, npts, pd, u ? ud : nullptr, du ? ud + npts : nullptr));
+  CK(k_field(h, npts, pd, u ? ud : nullptr, du ? ud + npts : nullptr, by_tree));
   if (u)
     CK(cudaMemcpyAsync(u, ud, sizeof(cplx) * npts, is_device_ptr(u) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                        h->stream));
@@ -2766,7 +2768,7 @@ pfmbem_status pfmbem_etc(pfmbem_t h, const double* psi, double x1, int npts, dou
     pts[2 * i + 1] = h->y0 + h->H * (i + 0.5) / npts;
   }
   std::vector<cplx> du(npts);
-  pfmbem_status st = field_points(h, psi, npts, pts.data(), nullptr, reinterpret_cast<double*>(du.data()));
+  pfmbem_status st = field_points(h, psi, npts, pts.data(), nullptr, reinterpret_cast<double*>(du.data()), true);
   if (st != PFMBEM_OK) return st;
   const double c = std::cos(h->theta), s = std::sin(h->theta);
   double sum = 0;

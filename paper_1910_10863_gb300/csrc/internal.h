@@ -194,6 +194,7 @@ struct pfmbem {
   cplx* self4 = nullptr;         // [E][4]: S_ee(k), T_ee(k), S_ee(k1), T_ee(k1)
   std::vector<int> hfib_off;
   int max_fiber = 0;
+  double hmax = 0;               // longest element
   // near lists over non-empty leaves (CSR): source leaf, image m
   int* nl_ptr = nullptr;
   int* nl_src = nullptr;
@@ -457,7 +458,7 @@ cudaError_t k_tri_l2l_dd(pfmbem* h, int l);
 cudaError_t k_wide_local(pfmbem* h);
 cudaError_t k_matvec(pfmbem* h, const cplx* x, cplx* y, int precision);
 cudaError_t k_rhs(pfmbem* h, cplx* B);
-cudaError_t k_field(pfmbem* h, const cplx* psi, int npts, const double2* pts, cplx* u, cplx* dudx1);
+cudaError_t k_field(pfmbem* h, int npts, const double2* pts, cplx* u, cplx* dudx1, bool by_tree);
 // BLAS-1 style helpers for GMRES (complex128, length n)
 cudaError_t k_multidot(pfmbem* h, const cplx* V, int ncol, const cplx* w, int n, cplx* out);
 cudaError_t k_gemv_sub(pfmbem* h, const cplx* V, int ncol, const cplx* coef, cplx* w, int n);
