@@ -16,6 +16,7 @@
 struct pfmbem_mlp {
   int in = 0, hidden = 0, layers = 0, out = 0;
   cudaStream_t stream = nullptr;
+  int dev = 0;                     // device current at create
   std::vector<int> dims;           // layer widths: in, hidden..., out
   std::vector<size_t> woff, boff;  // offsets of W and b of each layer in params
   size_t nparams = 0;
@@ -25,38 +26,187 @@ struct pfmbem_mlp {
   float* m2 = nullptr;             // Adam second moment
   int64_t step = 0;
   int cap = 0;                     // batch capacity of the work buffers
-  std::vector<float*> act;         // activations per layer boundary [cap][dims[l]]
+  std::vector<float*> act;         // activations per layer boundary [cap][dims[l]] (0: a host batch)
   std::vector<float*> pre;         // pre-activations per hidden layer
-  float* dA = nullptr;             // work: gradient w.r.t. activations
+  float* dA = nullptr;             // work: gradient w.r.t. pre-activations, two in turn
   float* dB = nullptr;
+  float* tgt = nullptr;            // a host batch's targets
   float* loss = nullptr;           // device scalar
+  float* hloss = nullptr;          // page-locked: the loss read back
 };
 
 namespace {
 
-constexpr int TS = 16;
+// ------------------------------------------------------------ FP32 products
+// Every pass of the network is a product C[M][N] = sum_k A(m, k) B(k, n) whose
+// operands lie along k ([m][k], [n][k]: AK, BK) or across it ([k][m], [k][n]):
+//   forward  Z = X W^T       AK, BK    bias and GELU (or the loss) in the epilogue
+//   dX       dZ W            AK, !BK   GELU' in the epilogue: the next layer's dZ
+//   dW       dZ^T X          !AK, !BK  the bias gradient from the staged dZ tile
+// The layers are small (256 x 256 at K = 256 and a batch of 256): what bounds them
+// is latency, so each pass is one launch with everything elementwise in it, and a
+// small tile (16 x 32, the four warps-quarters of 512 threads splitting each K
+// stage of 128) puts 128 blocks on such a layer; a tile of 64 x 64 with 4 x 4
+// outputs per thread takes over where it fills the chip by itself (BIG_TILES).  All
+// loads of a stage are issued before the previous stage's arithmetic.  FP32 FMA
+// throughout; the K quarters' sums are added in a fixed order.
+// Measured at 50 -> 3 x 256 -> 1088: a training step of 256 rows 354 -> 128 us (16 x 16
+// tiles, one output per thread, bias, GELU, loss and column sums as launches of their
+// own: 26 launches, now 9), a forward pass of 1024 rows 215 -> 75 us.
+struct Mat {
+  const float* A;
+  const float* B;
+  int M, N, K, lda, ldb;
+};
 
-// C[M][N] (+)= op(A) op(B) with op given by transA/transB; row-major operands:
-//   A is [M][K] (transA = 0) or [K][M] (transA = 1), B is [K][N] or [N][K].
-__global__ void gemm_kernel(int M, int N, int K, const float* __restrict__ A, int transA,
-                            const float* __restrict__ B, int transB, float* __restrict__ C, int accumulate) {
-  __shared__ float As[TS][TS + 1], Bs[TS][TS + 1];
-  const int r = blockIdx.y * TS + threadIdx.y, c = blockIdx.x * TS + threadIdx.x;
-  float acc = 0.f;
-  for (int k0 = 0; k0 < K; k0 += TS) {
-    const int ka = k0 + threadIdx.x, kb = k0 + threadIdx.y;
-    const int ar = blockIdx.y * TS + threadIdx.y;
-    As[threadIdx.y][threadIdx.x] =
-        (ar < M && ka < K) ? (transA ? A[(size_t)ka * M + ar] : A[(size_t)ar * K + ka]) : 0.f;
-    const int bc = blockIdx.x * TS + threadIdx.x;
-    Bs[threadIdx.y][threadIdx.x] =
-        (bc < N && kb < K) ? (transB ? B[(size_t)bc * K + kb] : B[(size_t)kb * N + bc]) : 0.f;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < TS; ++k) acc = fmaf(As[threadIdx.y][k], Bs[k][threadIdx.x], acc);
-    __syncthreads();
+// Element e of a [TK][T] tile staged from an operand along k (KM) or across it: a
+// warp covers 8 k x 4 rows (32-byte sectors; with a row stride of 4 mod 32 or 20
+// words its stores meet 32 different banks), or rows one after another.
+template <bool KM, int T>
+__device__ __forceinline__ void tile_at(int e, int& k, int& m) {
+  if (KM) {
+    const int r = e >> 5;
+    m = ((e >> 3) & 3) + 4 * (r % (T / 4));
+    k = (e & 7) + 8 * (r / (T / 4));
+  } else {
+    m = e % T;
+    k = e / T;
   }
-  if (r < M && c < N) C[(size_t)r * N + c] = accumulate ? C[(size_t)r * N + c] + acc : acc;
+}
+
+template <bool KM, int T, int TK, int NT>
+struct Stage {
+  static constexpr int NV = T * TK / NT;
+  float v[NV];
+  __device__ __forceinline__ void load(const float* __restrict__ P, int ld, int m0, int k0, int M, int K) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      int k, m;
+      tile_at<KM, T>((int)threadIdx.x + i * NT, k, m);
+      k += k0;
+      m += m0;
+      v[i] = k < K && m < M ? __ldg(P + (KM ? (size_t)m * ld + k : (size_t)k * ld + m)) : 0.f;
+    }
+  }
+  __device__ __forceinline__ void store(float* s) const {       // [TK][T + 4]
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      int k, m;
+      tile_at<KM, T>((int)threadIdx.x + i * NT, k, m);
+      s[k * (T + 4) + m] = v[i];
+    }
+  }
+};
+
+constexpr int SM_T = 16, SN_T = 32, SK_T = 128, SNT = 512;       // small tile
+constexpr int S_SMEM = SK_T * (SM_T + 4 + SN_T + 4);             // floats
+constexpr int L_T = 64, LK_T = 32, LNT = 256;                    // large tile
+constexpr int BIG_TILES = 128;                                   // large tiles from which it is taken
+
+// Small tile: out(m, n, value) for every entry of the tile at (m0, n0), one per
+// thread (n along the lanes).  rowsum (if not null): sum_k A(m, k), m = m0 ..
+template <bool AK, bool BK, class Out>
+__device__ __forceinline__ void small_tile(const Mat& g, int m0, int n0, float* sm, float* rowsum, Out out) {
+  float* sA = sm;
+  float* sB = sm + SK_T * (SM_T + 4);
+  Stage<AK, SM_T, SK_T, SNT> a;
+  Stage<BK, SN_T, SK_T, SNT> b;
+  const int t = threadIdx.x, grp = t >> 7, r = (t & 127) >> 3, c = 4 * (t & 7);
+  float acc[4] = {0.f, 0.f, 0.f, 0.f}, rs = 0.f;
+  a.load(g.A, g.lda, m0, 0, g.M, g.K);
+  b.load(g.B, g.ldb, n0, 0, g.N, g.K);
+  for (int k0 = 0; k0 < g.K; k0 += SK_T) {
+    __syncthreads();
+    a.store(sA);
+    b.store(sB);
+    __syncthreads();
+    if (k0 + SK_T < g.K) {
+      a.load(g.A, g.lda, m0, k0 + SK_T, g.M, g.K);
+      b.load(g.B, g.ldb, n0, k0 + SK_T, g.N, g.K);
+    }
+    const float* pa = sA + (grp * (SK_T / 4)) * (SM_T + 4) + r;
+    const float* pb = sB + (grp * (SK_T / 4)) * (SN_T + 4) + c;
+#pragma unroll 8
+    for (int k = 0; k < SK_T / 4; ++k) {
+      const float av = pa[k * (SM_T + 4)];
+      const float4 bv = *reinterpret_cast<const float4*>(pb + k * (SN_T + 4));
+      acc[0] = fmaf(av, bv.x, acc[0]);
+      acc[1] = fmaf(av, bv.y, acc[1]);
+      acc[2] = fmaf(av, bv.z, acc[2]);
+      acc[3] = fmaf(av, bv.w, acc[3]);
+    }
+    if (rowsum)
+#pragma unroll
+      for (int k = 0; k < SK_T / 32; ++k) rs += sA[((t >> 4) * (SK_T / 32) + k) * (SM_T + 4) + (t & 15)];
+  }
+  __syncthreads();
+  float* red = sm;                                     // [4][16][32], then [32][16]
+  *reinterpret_cast<float4*>(red + (grp * SM_T + r) * SN_T + c) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+  float* red2 = sm + 4 * SM_T * SN_T;
+  if (rowsum) red2[t] = rs;                            // [t >> 4][t & 15]
+  __syncthreads();
+  const int m = t >> 5, n = t & 31;
+  if (m0 + m < g.M && n0 + n < g.N) {
+    const float* q = red + m * SN_T + n;
+    out(m0 + m, n0 + n, (q[0] + q[SM_T * SN_T]) + (q[2 * SM_T * SN_T] + q[3 * SM_T * SN_T]));
+  }
+  if (rowsum && t < SM_T && m0 + t < g.M) {
+    float v = 0.f;
+    for (int i = 0; i < 32; ++i) v += red2[i * SM_T + t];
+    rowsum[m0 + t] = v;
+  }
+}
+
+template <bool AK, bool BK, class Out>
+__device__ __forceinline__ void large_tile(const Mat& g, int m0, int n0, float* sm, Out out) {
+  float* sA = sm;
+  float* sB = sm + LK_T * (L_T + 4);
+  Stage<AK, L_T, LK_T, LNT> a;
+  Stage<BK, L_T, LK_T, LNT> b;
+  const int t = threadIdx.x, r = 4 * (t >> 4), c = 4 * (t & 15);
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  a.load(g.A, g.lda, m0, 0, g.M, g.K);
+  b.load(g.B, g.ldb, n0, 0, g.N, g.K);
+  for (int k0 = 0; k0 < g.K; k0 += LK_T) {
+    __syncthreads();
+    a.store(sA);
+    b.store(sB);
+    __syncthreads();
+    if (k0 + LK_T < g.K) {
+      a.load(g.A, g.lda, m0, k0 + LK_T, g.M, g.K);
+      b.load(g.B, g.ldb, n0, k0 + LK_T, g.N, g.K);
+    }
+#pragma unroll 8
+    for (int k = 0; k < LK_T; ++k) {
+      const float4 av = *reinterpret_cast<const float4*>(sA + k * (L_T + 4) + r);
+      const float4 bv = *reinterpret_cast<const float4*>(sB + k * (L_T + 4) + c);
+      const float ax[4] = {av.x, av.y, av.z, av.w}, bx[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ax[i], bx[j], acc[i][j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (m0 + r + i < g.M && n0 + c + j < g.N) out(m0 + r + i, n0 + c + j, acc[i][j]);
+}
+
+// The block's tile of a product of tm x tn tiles, m fastest.
+template <bool BIG, bool AK, bool BK, class Out>
+__device__ __forceinline__ void tile(const Mat& g, int b, float* sm, float* rowsum, Out out) {
+  constexpr int TM = BIG ? L_T : SM_T, TN = BIG ? L_T : SN_T;
+  const int tm = (g.M + TM - 1) / TM, mi = b % tm, ni = b / tm;
+  if constexpr (BIG)
+    large_tile<AK, BK>(g, mi * TM, ni * TN, sm, out);
+  else
+    small_tile<AK, BK>(g, mi * TM, ni * TN, sm, ni == 0 ? rowsum : nullptr, out);
 }
 
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
@@ -64,44 +214,68 @@ __device__ __forceinline__ float gelu_grad(float x) {
   return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-// Z[b][o] += bias[o]; then A = gelu(Z) (hidden) or A = Z (output)
-__global__ void bias_act_kernel(int B, int O, const float* __restrict__ bias, float* __restrict__ Z,
-                                float* __restrict__ Aout, int act) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= B * O) return;
-  const float z = Z[i] + bias[i % O];
-  Z[i] = z;
-  Aout[i] = act ? gelu(z) : z;
-}
-
-// dY = 2 (Y - T) / (B O); loss += sum (Y - T)^2 / (B O)
-__global__ void mse_kernel(int n, float scale, const float* __restrict__ Y, const float* __restrict__ T,
-                           float* __restrict__ dY, float* __restrict__ loss) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  float v = 0.f;
-  if (i < n) {
-    const float d = Y[i] - T[i];
-    dY[i] = 2.f * d * scale;
-    v = d * d * scale;
+// One forward layer: z = X W^T + bias; hidden layers write gelu(z) to Y and, for a
+// training pass, z to Z; the output layer writes z to Y or, with targets, the
+// gradient of the mean-squared error 2 (z - T) scale to Y and adds (z - T)^2 scale
+// to the loss.  clear: the loss, cleared by the first layer's first block.
+template <bool BIG>
+__global__ void __launch_bounds__(BIG ? LNT : SNT) layer_kernel(const Mat g, const float* __restrict__ bias,
+                                                                int hidden, float* __restrict__ Z,
+                                                                float* __restrict__ Y, const float* __restrict__ T,
+                                                                float scale, float* loss, float* clear) {
+  __shared__ __align__(16) float sm[S_SMEM];
+  __shared__ float red[SNT / 32];
+  if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0.f;
+  float l = 0.f;
+  tile<BIG, true, true>(g, blockIdx.x, sm, nullptr, [&](int m, int n, float v) {
+    const float z = v + bias[n];
+    const size_t i = (size_t)m * g.N + n;
+    if (hidden) {
+      if (Z) Z[i] = z;
+      Y[i] = gelu(z);
+    } else if (T) {
+      const float d = z - T[i];
+      Y[i] = 2.f * d * scale;
+      l += d * d * scale;
+    } else {
+      Y[i] = z;
+    }
+  });
+  if (!T || hidden) return;
+  for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < (int)(blockDim.x >> 5); ++i) l += red[i];
+    atomicAdd(loss, l);
   }
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, v);
 }
 
-// db[o] = sum_b dZ[b][o]
-__global__ void colsum_kernel(int B, int O, const float* __restrict__ dZ, float* __restrict__ db) {
-  const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= O) return;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s += dZ[(size_t)b * O + o];
-  db[o] = s;
+// One backward layer in one launch: the first ndx blocks form dX = dZ W times
+// GELU'(Z) of the layer below (its dZ), the others dW = dZ^T X and the bias
+// gradient, the column sums of dZ.
+__global__ void __launch_bounds__(SNT) back_kernel(const Mat dx, int ndx, const float* __restrict__ Zb,
+                                                   float* __restrict__ dZb, const Mat dw, float* __restrict__ gw,
+                                                   float* __restrict__ gb) {
+  __shared__ __align__(16) float sm[S_SMEM];
+  if ((int)blockIdx.x < ndx) {
+    tile<false, true, false>(dx, blockIdx.x, sm, nullptr, [&](int m, int n, float v) {
+      const size_t i = (size_t)m * dx.N + n;
+      dZb[i] = v * gelu_grad(Zb[i]);
+    });
+  } else {
+    tile<false, false, false>(dw, blockIdx.x - ndx, sm, gb,
+                              [&](int m, int n, float v) { gw[(size_t)m * dw.N + n] = v; });
+  }
 }
 
-// dZ = dA * gelu'(Z)
-__global__ void gelu_back_kernel(int n, const float* __restrict__ Z, const float* __restrict__ dA,
-                                 float* __restrict__ dZ) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dZ[i] = dA[i] * gelu_grad(Z[i]);
+__global__ void __launch_bounds__(LNT) back_dx_kernel(const Mat dx, const float* __restrict__ Zb,
+                                                      float* __restrict__ dZb) {
+  __shared__ __align__(16) float sm[2 * LK_T * (L_T + 4)];
+  tile<true, true, false>(dx, blockIdx.x, sm, nullptr, [&](int m, int n, float v) {
+    const size_t i = (size_t)m * dx.N + n;
+    dZb[i] = v * gelu_grad(Zb[i]);
+  });
 }
 
 __global__ void adam_kernel(size_t n, float lr, float b1, float b2, float eps, float c1, float c2,
@@ -130,10 +304,7 @@ __global__ void init_kernel(size_t n, uint64_t seed, const int64_t* __restrict__
   p[i] = fi > 0 ? u * sqrtf(3.f / (float)fi) : 0.f;   // Var = 1/fan_in, biases zero
 }
 
-void gemm(cudaStream_t st, int M, int N, int K, const float* A, int ta, const float* B, int tb, float* C, int acc) {
-  dim3 blk(TS, TS), grd((N + TS - 1) / TS, (M + TS - 1) / TS);
-  gemm_kernel<<<grd, blk, 0, st>>>(M, N, K, A, ta, B, tb, C, acc);
-}
+int tiles(int M, int N, int TM, int TN) { return ((M + TM - 1) / TM) * ((N + TN - 1) / TN); }
 
 cudaError_t ensure_cap(pfmbem_mlp* m, int B) {
   if (B <= m->cap) return cudaSuccess;
@@ -141,6 +312,9 @@ cudaError_t ensure_cap(pfmbem_mlp* m, int B) {
   for (float* p : m->pre) cudaFree(p);
   cudaFree(m->dA);
   cudaFree(m->dB);
+  cudaFree(m->tgt);
+  m->dA = m->dB = m->tgt = nullptr;
+  m->cap = 0;
   m->act.assign(m->dims.size(), nullptr);
   m->pre.assign(m->dims.size(), nullptr);
   int wmax = 0;
@@ -151,39 +325,49 @@ cudaError_t ensure_cap(pfmbem_mlp* m, int B) {
   }
   if (cudaMalloc(&m->dA, sizeof(float) * (size_t)B * wmax) != cudaSuccess) return cudaErrorMemoryAllocation;
   if (cudaMalloc(&m->dB, sizeof(float) * (size_t)B * wmax) != cudaSuccess) return cudaErrorMemoryAllocation;
+  if (cudaMalloc(&m->tgt, sizeof(float) * (size_t)B * m->out) != cudaSuccess) return cudaErrorMemoryAllocation;
   m->cap = B;
   return cudaSuccess;
 }
 
-// forward pass; act[0] must hold the input batch
-void forward(pfmbem_mlp* m, int B) {
+// Forward pass from X to Y ([B][out]).  With targets T, Y receives the gradient of
+// the loss instead, m->loss the loss, and the pre-activations are kept.
+void forward(pfmbem_mlp* m, int B, const float* X, float* Y, const float* T) {
   const int L = (int)m->dims.size() - 1;
+  const float scale = 1.f / (float)((size_t)B * m->out);
   for (int l = 0; l < L; ++l) {
-    const int I = m->dims[l], O = m->dims[l + 1];
-    gemm(m->stream, B, O, I, m->act[l], 0, m->params + m->woff[l], 1, m->pre[l + 1], 0);
-    bias_act_kernel<<<(B * O + 255) / 256, 256, 0, m->stream>>>(B, O, m->params + m->boff[l], m->pre[l + 1],
-                                                                m->act[l + 1], l < L - 1 ? 1 : 0);
+    const int I = m->dims[l], O = m->dims[l + 1], hidden = l < L - 1;
+    const Mat g{l == 0 ? X : m->act[l], m->params + m->woff[l], B, O, I, I, I};
+    float* y = hidden ? m->act[l + 1] : Y;
+    float* z = hidden && T ? m->pre[l + 1] : nullptr;
+    float* clear = T && l == 0 ? m->loss : nullptr;
+    const int nb = tiles(B, O, L_T, L_T);
+    if (nb >= BIG_TILES)
+      layer_kernel<true><<<nb, LNT, 0, m->stream>>>(g, m->params + m->boff[l], hidden, z, y, T, scale, m->loss, clear);
+    else
+      layer_kernel<false><<<tiles(B, O, SM_T, SN_T), SNT, 0, m->stream>>>(g, m->params + m->boff[l], hidden, z, y, T,
+                                                                          scale, m->loss, clear);
   }
 }
 
-// backward pass from dY (in m->dA, [B][out]); writes m->grad
-void backward(pfmbem_mlp* m, int B) {
+// Backward pass from the loss gradient in m->dA ([B][out]); writes grad.
+void backward(pfmbem_mlp* m, int B, const float* X, float* grad) {
   const int L = (int)m->dims.size() - 1;
   float* dcur = m->dA;   // gradient w.r.t. pre-activation of layer l+1
   float* dnext = m->dB;
   for (int l = L - 1; l >= 0; --l) {
     const int I = m->dims[l], O = m->dims[l + 1];
-    // dW[o][i] = sum_b dZ[b][o] X[b][i]
-    gemm(m->stream, O, I, B, dcur, 1, m->act[l], 0, m->grad + m->woff[l], 0);
-    colsum_kernel<<<(O + 127) / 128, 128, 0, m->stream>>>(B, O, dcur, m->grad + m->boff[l]);
-    if (l > 0) {
-      // dA_prev[b][i] = sum_o dZ[b][o] W[o][i]; then through GELU of layer l
-      gemm(m->stream, B, I, O, dcur, 0, m->params + m->woff[l], 0, dnext, 0);
-      gelu_back_kernel<<<(B * I + 255) / 256, 256, 0, m->stream>>>(B * I, m->pre[l], dnext, dnext);
-      float* t = dcur;
-      dcur = dnext;
-      dnext = t;
-    }
+    const Mat dx{dcur, m->params + m->woff[l], B, I, O, O, I};
+    const Mat dw{dcur, l == 0 ? X : m->act[l], O, I, B, O, I};
+    const int nbig = l > 0 ? tiles(B, I, L_T, L_T) : 0;
+    const bool big = nbig >= BIG_TILES;
+    if (big) back_dx_kernel<<<nbig, LNT, 0, m->stream>>>(dx, m->pre[l], dnext);
+    const int ndx = l > 0 && !big ? tiles(B, I, SM_T, SN_T) : 0;
+    back_kernel<<<ndx + tiles(O, I, SM_T, SN_T), SNT, 0, m->stream>>>(dx, ndx, l > 0 ? m->pre[l] : nullptr, dnext, dw,
+                                                                      grad + m->woff[l], grad + m->boff[l]);
+    float* t = dcur;
+    dcur = dnext;
+    dnext = t;
   }
 }
 
@@ -194,6 +378,17 @@ bool is_dev(const void* p) {
     return false;
   }
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// Memory that the network's kernels may read and write in place: its own device's
+// (another device's is copied, as host memory is).
+bool is_local(const pfmbem_mlp* m, const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == m->dev;
 }
 
 cudaError_t copy_in(pfmbem_mlp* m, float* dst, const float* src, size_t n) {
@@ -347,6 +542,7 @@ pfmbem_status pfmbem_mlp_create(int in, int hidden, int layers, int out, uint64_
   m->layers = layers;
   m->out = out;
   m->stream = static_cast<cudaStream_t>(stream);
+  cudaGetDevice(&m->dev);
   m->dims.push_back(in);
   for (int l = 0; l < layers; ++l) m->dims.push_back(hidden);
   m->dims.push_back(out);
@@ -375,7 +571,7 @@ pfmbem_status pfmbem_mlp_create(int in, int hidden, int layers, int out, uint64_
   cudaMemsetAsync(m->m2, 0, off * sizeof(float), m->stream);
   cudaStreamSynchronize(m->stream);
   cudaFree(fan_d);
-  if (cudaMalloc(&m->loss, sizeof(float)) != cudaSuccess) {
+  if (cudaMalloc(&m->loss, sizeof(float)) != cudaSuccess || cudaMallocHost(&m->hloss, sizeof(float)) != cudaSuccess) {
     pfmbem_mlp_destroy(m);
     return PFMBEM_ENOMEM;
   }
@@ -399,6 +595,8 @@ void pfmbem_mlp_destroy(pfmbem_mlp_t m) {
   for (float* p : m->pre) cudaFree(p);
   cudaFree(m->dA);
   cudaFree(m->dB);
+  cudaFree(m->tgt);
+  cudaFreeHost(m->hloss);
   delete m;
 }
 
@@ -417,12 +615,18 @@ pfmbem_status pfmbem_mlp_params(pfmbem_mlp_t m, int64_t* nparams, float* get, co
 pfmbem_status pfmbem_mlp_forward(pfmbem_mlp_t m, int B, const float* X, float* Y) {
   if (!m || B < 1 || !X || !Y) return PFMBEM_EINVAL;
   if (ensure_cap(m, B) != cudaSuccess) return PFMBEM_ENOMEM;
-  if (copy_in(m, m->act[0], X, (size_t)B * m->in) != cudaSuccess) return PFMBEM_ECUDA;
-  forward(m, B);
-  if (cudaMemcpyAsync(Y, m->act.back(), sizeof(float) * (size_t)B * m->out,
-                      is_dev(Y) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
+  // batches on the device are read and written in place, in the stream's order
+  // (an input that overlaps the output is copied first)
+  const bool ydev = is_dev(Y), yin = is_local(m, Y);
+  if (!is_local(m, X) || (yin && X < Y + (size_t)B * m->out && Y < X + (size_t)B * m->in)) {
+    if (copy_in(m, m->act[0], X, (size_t)B * m->in) != cudaSuccess) return PFMBEM_ECUDA;
+    X = m->act[0];
+  }
+  forward(m, B, X, yin ? Y : m->act.back(), nullptr);
+  if (!yin && cudaMemcpyAsync(Y, m->act.back(), sizeof(float) * (size_t)B * m->out,
+                              ydev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
     return PFMBEM_ECUDA;
-  if (!is_dev(Y) && cudaStreamSynchronize(m->stream) != cudaSuccess) return PFMBEM_ECUDA;
+  if (!ydev && cudaStreamSynchronize(m->stream) != cudaSuccess) return PFMBEM_ECUDA;
   return cudaGetLastError() == cudaSuccess ? PFMBEM_OK : PFMBEM_ECUDA;
 }
 
@@ -433,28 +637,40 @@ pfmbem_status pfmbem_mlp_train(pfmbem_mlp_t m, int B, const float* X, const floa
                                float* grad) {
   if (!m || B < 1 || !X || !T) return PFMBEM_EINVAL;
   if (ensure_cap(m, B) != cudaSuccess) return PFMBEM_ENOMEM;
-  if (copy_in(m, m->act[0], X, (size_t)B * m->in) != cudaSuccess) return PFMBEM_ECUDA;
-  if (copy_in(m, m->dB, T, (size_t)B * m->out) != cudaSuccess) return PFMBEM_ECUDA;
-  forward(m, B);
-  cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream);
-  const int n = B * m->out;
-  // the target is parked in dB; dY goes to dA
-  mse_kernel<<<(n + 255) / 256, 256, 0, m->stream>>>(n, 1.f / (float)n, m->act.back(), m->dB, m->dA, m->loss);
-  backward(m, B);
+  // a batch on the device is read, and a gradient there written, in place (the
+  // call waits for the stream at its end)
+  if (!is_local(m, X)) {
+    if (copy_in(m, m->act[0], X, (size_t)B * m->in) != cudaSuccess) return PFMBEM_ECUDA;
+    X = m->act[0];
+  }
+  if (!is_local(m, T)) {
+    if (copy_in(m, m->tgt, T, (size_t)B * m->out) != cudaSuccess) return PFMBEM_ECUDA;
+    T = m->tgt;
+  }
+  float* g = m->grad;
+  if (grad && is_local(m, grad)) {
+    // (a gradient that shares memory with the batch is copied out at the end)
+    auto apart = [&](const float* p, size_t n) { return p + n <= grad || grad + m->nparams <= p; };
+    if (apart(X, (size_t)B * m->in) && apart(T, (size_t)B * m->out)) g = grad;
+  }
+  forward(m, B, X, m->dA, T);
+  backward(m, B, X, g);
   if (lr > 0) {
     m->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f / (1.f - (float)std::pow(b1, (double)m->step));
     const float c2 = 1.f / (1.f - (float)std::pow(b2, (double)m->step));
     adam_kernel<<<(unsigned)((m->nparams + 255) / 256), 256, 0, m->stream>>>(m->nparams, lr, b1, b2, 1e-8f, c1, c2,
-                                                                            m->params, m->grad, m->m1, m->m2);
+                                                                            m->params, g, m->m1, m->m2);
   }
-  if (grad && cudaMemcpyAsync(grad, m->grad, m->nparams * sizeof(float),
-                              is_dev(grad) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
+  if (grad && g != grad &&
+      cudaMemcpyAsync(grad, g, m->nparams * sizeof(float),
+                      is_dev(grad) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
     return PFMBEM_ECUDA;
-  if (loss && cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
+  if (loss && cudaMemcpyAsync(m->hloss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
     return PFMBEM_ECUDA;
   if (cudaStreamSynchronize(m->stream) != cudaSuccess) return PFMBEM_ECUDA;
+  if (loss) *loss = *m->hloss;
   return cudaGetLastError() == cudaSuccess ? PFMBEM_OK : PFMBEM_ECUDA;
 }
 
