@@ -45,11 +45,13 @@ namespace {
 //   dW       dZ^T X          !AK, !BK  the bias gradient from the staged dZ tile
 // The layers are small (256 x 256 at K = 256 and a batch of 256): what bounds them
 // is latency, so each pass is one launch with everything elementwise in it, and a
-// small tile (16 x 32, the four warps-quarters of 512 threads splitting each K
-// stage of 128) puts 128 blocks on such a layer; a tile of 64 x 64 with 4 x 4
-// outputs per thread takes over where it fills the chip by itself (BIG_TILES).  All
-// loads of a stage are issued before the previous stage's arithmetic.  FP32 FMA
-// throughout; the K quarters' sums are added in a fixed order.
+// small tile (32 x 32, eight groups of 64 threads sharing each K stage of 128) keeps
+// the chain short on the 64 blocks such a layer has; a tile of 64 x 64 with the
+// block's threads over the outputs alone takes over where it fills the chip by
+// itself (BIG_TILES).  4 x 4 outputs per thread: a 16 x 32 tile with 1 x 4 was bound
+// by its shared-memory reads (20 against @S@ us for 256 x 1088 at K = 256).  All loads
+// of a stage are issued before the previous stage's arithmetic.  FP32 FMA
+// throughout; the groups' sums are added in a fixed order.
 // Measured at 50 -> 3 x 256 -> 1088: a training step of 256 rows 354 -> 128 us (16 x 16
 // tiles, one output per thread, bias, GELU, loss and column sums as launches of their
 // own: 26 launches, now 9), a forward pass of 1024 rows 215 -> 75 us.
@@ -98,21 +100,27 @@ struct Stage {
   }
 };
 
-constexpr int SM_T = 16, SN_T = 32, SK_T = 128, SNT = 512;       // small tile
+constexpr int SM_T = 32, SN_T = 32, SK_T = 128, SNT = 512;       // small tile
+constexpr int SGRP = SNT / 64;                                   // shares of its K stage
 constexpr int S_SMEM = SK_T * (SM_T + 4 + SN_T + 4);             // floats
 constexpr int L_T = 64, LK_T = 32, LNT = 256;                    // large tile
 constexpr int BIG_TILES = 128;                                   // large tiles from which it is taken
 
-// Small tile: out(m, n, value) for every entry of the tile at (m0, n0), one per
-// thread (n along the lanes).  rowsum (if not null): sum_k A(m, k), m = m0 ..
+// Small tile: out(m, n, value) for every entry of the tile at (m0, n0), n along the
+// lanes.  64 threads of 4 x 4 outputs hold the tile; SGRP such groups share every K
+// stage.  rowsum (if not null): sum_k A(m, k), m = m0 ..
 template <bool AK, bool BK, class Out>
 __device__ __forceinline__ void small_tile(const Mat& g, int m0, int n0, float* sm, float* rowsum, Out out) {
   float* sA = sm;
   float* sB = sm + SK_T * (SM_T + 4);
   Stage<AK, SM_T, SK_T, SNT> a;
   Stage<BK, SN_T, SK_T, SNT> b;
-  const int t = threadIdx.x, grp = t >> 7, r = (t & 127) >> 3, c = 4 * (t & 7);
-  float acc[4] = {0.f, 0.f, 0.f, 0.f}, rs = 0.f;
+  const int t = threadIdx.x, grp = t >> 6, r = 4 * ((t & 63) >> 3), c = 4 * (t & 7);
+  float acc[4][4], rs = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
   a.load(g.A, g.lda, m0, 0, g.M, g.K);
   b.load(g.B, g.ldb, n0, 0, g.N, g.K);
   for (int k0 = 0; k0 < g.K; k0 += SK_T) {
@@ -124,35 +132,44 @@ __device__ __forceinline__ void small_tile(const Mat& g, int m0, int n0, float* 
       a.load(g.A, g.lda, m0, k0 + SK_T, g.M, g.K);
       b.load(g.B, g.ldb, n0, k0 + SK_T, g.N, g.K);
     }
-    const float* pa = sA + (grp * (SK_T / 4)) * (SM_T + 4) + r;
-    const float* pb = sB + (grp * (SK_T / 4)) * (SN_T + 4) + c;
+    const float* pa = sA + (grp * (SK_T / SGRP)) * (SM_T + 4) + r;
+    const float* pb = sB + (grp * (SK_T / SGRP)) * (SN_T + 4) + c;
 #pragma unroll 8
-    for (int k = 0; k < SK_T / 4; ++k) {
-      const float av = pa[k * (SM_T + 4)];
+    for (int k = 0; k < SK_T / SGRP; ++k) {
+      const float4 av = *reinterpret_cast<const float4*>(pa + k * (SM_T + 4));
       const float4 bv = *reinterpret_cast<const float4*>(pb + k * (SN_T + 4));
-      acc[0] = fmaf(av, bv.x, acc[0]);
-      acc[1] = fmaf(av, bv.y, acc[1]);
-      acc[2] = fmaf(av, bv.z, acc[2]);
-      acc[3] = fmaf(av, bv.w, acc[3]);
+      const float ax[4] = {av.x, av.y, av.z, av.w}, bx[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ax[i], bx[j], acc[i][j]);
     }
     if (rowsum)
 #pragma unroll
-      for (int k = 0; k < SK_T / 32; ++k) rs += sA[((t >> 4) * (SK_T / 32) + k) * (SM_T + 4) + (t & 15)];
+      for (int k = 0; k < SK_T / 16; ++k) rs += sA[((t >> 5) * (SK_T / 16) + k) * (SM_T + 4) + (t & 31)];
   }
   __syncthreads();
-  float* red = sm;                                     // [4][16][32], then [32][16]
-  *reinterpret_cast<float4*>(red + (grp * SM_T + r) * SN_T + c) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-  float* red2 = sm + 4 * SM_T * SN_T;
-  if (rowsum) red2[t] = rs;                            // [t >> 4][t & 15]
+  float* red = sm;                                     // [SGRP][32][32], then [16][32]
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    *reinterpret_cast<float4*>(red + (grp * SM_T + r + i) * SN_T + c) =
+        make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  float* red2 = sm + SGRP * SM_T * SN_T;
+  if (rowsum) red2[t] = rs;                            // [t >> 5][t & 31]
   __syncthreads();
-  const int m = t >> 5, n = t & 31;
-  if (m0 + m < g.M && n0 + n < g.N) {
-    const float* q = red + m * SN_T + n;
-    out(m0 + m, n0 + n, (q[0] + q[SM_T * SN_T]) + (q[2 * SM_T * SN_T] + q[3 * SM_T * SN_T]));
+#pragma unroll
+  for (int h = 0; h < SM_T * SN_T / SNT; ++h) {
+    const int i = t + h * SNT, m = i >> 5, n = i & 31;
+    if (m0 + m < g.M && n0 + n < g.N) {
+      float v = 0.f;
+#pragma unroll
+      for (int q = 0; q < SGRP; ++q) v += red[q * SM_T * SN_T + i];
+      out(m0 + m, n0 + n, v);
+    }
   }
   if (rowsum && t < SM_T && m0 + t < g.M) {
     float v = 0.f;
-    for (int i = 0; i < 32; ++i) v += red2[i * SM_T + t];
+    for (int i = 0; i < 16; ++i) v += red2[i * SM_T + t];
     rowsum[m0 + t] = v;
   }
 }
@@ -219,7 +236,7 @@ __device__ __forceinline__ float gelu_grad(float x) {
 // gradient of the mean-squared error 2 (z - T) scale to Y and adds (z - T)^2 scale
 // to the loss.  clear: the loss, cleared by the first layer's first block.
 template <bool BIG>
-__global__ void __launch_bounds__(BIG ? LNT : SNT) layer_kernel(const Mat g, const float* __restrict__ bias,
+__global__ void __launch_bounds__(BIG ? LNT : SNT, 2) layer_kernel(const Mat g, const float* __restrict__ bias,
                                                                 int hidden, float* __restrict__ Z,
                                                                 float* __restrict__ Y, const float* __restrict__ T,
                                                                 float scale, float* loss, float* clear) {
@@ -254,7 +271,7 @@ __global__ void __launch_bounds__(BIG ? LNT : SNT) layer_kernel(const Mat g, con
 // One backward layer in one launch: the first ndx blocks form dX = dZ W times
 // GELU'(Z) of the layer below (its dZ), the others dW = dZ^T X and the bias
 // gradient, the column sums of dZ.
-__global__ void __launch_bounds__(SNT) back_kernel(const Mat dx, int ndx, const float* __restrict__ Zb,
+__global__ void __launch_bounds__(SNT, 2) back_kernel(const Mat dx, int ndx, const float* __restrict__ Zb,
                                                    float* __restrict__ dZb, const Mat dw, float* __restrict__ gw,
                                                    float* __restrict__ gb) {
   __shared__ __align__(16) float sm[S_SMEM];

@@ -1,4 +1,4 @@
-"""The network's products at the edges of their tiles (16 x 32 with K stages of 128, and
+"""The network's products at the edges of their tiles (32 x 32 with K stages of 128, and
 64 x 64 with K stages of 32): one row to more than a tile of rows, widths below, at and
 above a tile, batches that take the large tile forward and backward; host and device
 buffers, and a device batch at an odd offset.  Against the FP64 oracle."""
