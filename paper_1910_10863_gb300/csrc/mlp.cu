@@ -49,12 +49,13 @@ namespace {
 // the chain short on the 64 blocks such a layer has; a tile of 64 x 64 with the
 // block's threads over the outputs alone takes over where it fills the chip by
 // itself (BIG_TILES).  4 x 4 outputs per thread: a 16 x 32 tile with 1 x 4 was bound
-// by its shared-memory reads (20 against @S@ us for 256 x 1088 at K = 256).  All loads
+// by its shared-memory reads (20 against 15 us for 256 x 1088 at K = 256).  All loads
 // of a stage are issued before the previous stage's arithmetic.  FP32 FMA
 // throughout; the groups' sums are added in a fixed order.
 // Measured at 50 -> 3 x 256 -> 1088: a training step of 256 rows 354 -> 128 us (16 x 16
 // tiles, one output per thread, bias, GELU, loss and column sums as launches of their
-// own: 26 launches, now 9), a forward pass of 1024 rows 215 -> 75 us.
+// own: 26 launches, now 9), then 102 with 4 x 4 outputs a thread; a forward pass of 1024
+// rows 215 -> 57 us.
 struct Mat {
   const float* A;
   const float* B;
