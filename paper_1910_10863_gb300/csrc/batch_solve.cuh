@@ -494,7 +494,7 @@ cudaError_t batch_fill(pfmbem* h, int GS, FusedArgs<C>& a) {
     const int fb = (int)((double)GS * nf / (nf + wa) + 0.5);
     a.fblk = GS >= 16 ? std::max(1, std::min({fb, nf, GS - GS / 4})) : 0;
   }
-  a.m2l_warp = f32 ? 0 : 1;
+  a.m2l_warp = !f32 && !a.nc_lo;      // staged chunks but for an FP64 product without double-float tables
   a.near_first = 0;
   {
     const int64_t w = (int64_t)GS * FW;

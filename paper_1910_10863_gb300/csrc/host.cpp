@@ -1275,7 +1275,7 @@ static pfmbem_status build_plan(pfmbem* h, const int* npf, const double* nodes) 
       const size_t ex = up16((size_t)L.nbox * L.P);
       const size_t tm = l >= 1 ? up16((size_t)49 * L.P * L.P) : 0;
       const size_t mm = l < D ? up16((size_t)4 * L.P * h->lev[l + 1].P) : 0;
-      n64 += 2 * ex + 2 * tm + 2 * mm;
+      n64 += 3 * ex + 2 * tm + 2 * mm;
       n32 += 2 * up16(ex) + 3 * up16(tm) + 4 * up16(mm);
     }
     cplx* a64 = dalloc<cplx>(h, n64);
@@ -1288,6 +1288,7 @@ static pfmbem_status build_plan(pfmbem* h, const int* npf, const double* nodes) 
       const size_t ex = up16((size_t)L.nbox * P);
       L.M = a64; a64 += ex;
       L.L = a64; a64 += ex;
+      L.Mw = reinterpret_cast<float4*>(a64); a64 += ex;
       L.Mf = a32; a32 += ex;
       L.Lf = a32; a32 += ex;
       tl.p[l] = L.p;

@@ -82,6 +82,7 @@ struct Level {
   cplx* m2lt = nullptr;      // the same operators transposed, [49][P source][P target]
   cplxf* m2ltf = nullptr;
   cplxf* m2ltl = nullptr;    // lo parts of m2lt: m2lt = m2ltf + m2ltl to ~48 bits (double-float M2L)
+  float4* Mw = nullptr;      // multipoles as double-float words (hi.re, hi.im, lo.re, lo.im), FP64 single-launch product
   // triangle tree: box centres, and per box the index of its M2M/L2L operator in
   // the parent level's tables (the children's offsets vary with the orientation)
   double2* ctr = nullptr;    // [nbox]

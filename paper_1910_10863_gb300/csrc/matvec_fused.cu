@@ -158,6 +158,8 @@ struct FusedArgs {
   const cplxf* nc_lo;                // lo parts of the near blocks (hi parts: the FP32 copy)
   cplxf* dens_dd;                    // [2][2E] hi and lo parts of the sorted densities
   const cplxf* nc_hi;
+  float4* Mw[PF_MAXLEVEL + 1];           // FP64 product: the multipoles as double-float words, beside M
+  float4 alpha_w;                        // alpha as such a word
   const cplxf* m2lth[PF_MAXLEVEL + 1];   // FP64 product, double-float M2L: hi and lo parts of m2lt
   const cplxf* m2ltl[PF_MAXLEVEL + 1];
   const cplxf* m2mh[PF_MAXLEVEL + 1];    // FP64 product, double-float M2M: hi and lo parts of m2m
@@ -168,7 +170,6 @@ struct FusedArgs {
   const cplxf* l2ll[PF_MAXLEVEL + 1];
   const cplxf* l2ph;                     // FP64 product, double-float L2P: hi and lo parts of l2p
   const cplxf* l2pl;
-  int l2p_dd;                            // measurement (PFMBEM_L2P_DD=1): it measured slower than FP64
   // FP32 product: near-field sums in differences (dlo: lo parts of the sorted
   // densities, rsum: FP64 row sums of the near blocks) and the same-fiber FFTs
   // in FP64 (fh64, tw64: the FP64 block symbols and twiddles)
@@ -634,35 +635,90 @@ __device__ __forceinline__ dflt dd_wsum(dflt v) {
 
 __device__ __forceinline__ double dd_value(dflt v) { return (double)v.h + (double)v.l; }
 
+// A complex value's hi and lo parts as one 16-byte word (hi.re, hi.im, lo.re, lo.im),
+// the form in which the double-float sums keep vectors and operators in shared memory.
+__device__ __forceinline__ float4 dd_word(cplx v) {
+  const cplxf h = to_f(v), l = split_lo(v);
+  return make_float4(h.re, h.im, l.re, l.im);
+}
+__device__ __forceinline__ void dd_cmac(dflt& re, dflt& im, float4 a, float4 b) {
+  dd_cmac(re, im, cplxf{a.x, a.y}, cplxf{a.z, a.w}, cplxf{b.x, b.y}, cplxf{b.z, b.w});
+}
+// The word of a complex double-float sum (hi the rounding of hi + lo).
+__device__ __forceinline__ float4 dd_word(dflt re, dflt im) {
+  const float h = __fadd_rn(re.h, re.l), g = __fadd_rn(im.h, im.l);
+  return make_float4(h, g, __fadd_rn(re.l, __fsub_rn(re.h, h)), __fadd_rn(im.l, __fsub_rn(im.h, g)));
+}
+// alpha^m v for m in {-1, 0, 1}
+__device__ __forceinline__ float4 dd_phase(float4 al, int m, float4 v) {
+  if (m == 0) return v;
+  if (m < 0) {
+    al.y = -al.y;
+    al.w = -al.w;
+  }
+  dflt re{0, 0}, im{0, 0};
+  dd_cmac(re, im, al, v);
+  return dd_word(re, im);
+}
+// Sums over the warp of four double-float values: the lanes halve the values they
+// carry in the first two steps, so that it takes six additions instead of twenty.
+// On return lanes 0, 8, 16, 24 hold the sums of a, b, c, d.
+__device__ __forceinline__ dflt dd_wsum4(dflt a, dflt b, dflt c, dflt d, int lane) {
+  auto x = [](dflt v, int o) {
+    return dflt{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+  };
+  const bool u = (lane & 16) != 0, v = (lane & 8) != 0;
+  const dflt p = dd_add(u ? c : a, x(u ? a : c, 16)), q = dd_add(u ? d : b, x(u ? b : d, 16));
+  dflt r = dd_add(v ? q : p, x(v ? p : q, 8));
+  r = dd_add(r, x(r, 4));
+  r = dd_add(r, x(r, 2));
+  return dd_add(r, x(r, 1));
+}
+// re, im += sum_{m < K} T_m[n] w[m], operator rows of stride S from its hi and lo
+// tables (device memory, lanes over n), w in shared memory.
+__device__ __forceinline__ void dd_rows(dflt& re, dflt& im, const cplxf* __restrict__ Th, const cplxf* __restrict__ Tl,
+                                        int S, const float4* w, int K) {
+#pragma unroll 7
+  for (int m = 0; m < K; ++m) {
+    const float4 v = w[m];
+    dd_cmac(re, im, Th[(size_t)m * S], Tl[(size_t)m * S], cplxf{v.x, v.y}, cplxf{v.z, v.w});
+  }
+}
+
 // Near-field sum of one target (sorted element s) in double-float arithmetic:
 // the FP64 product's near field with FP32 instructions (GB300 issues FP64 at
-// 1/64 of the FP32 rate) and FP64-level accuracy.  Writes the FP64 Un of s.
+// 1/64 of the FP32 rate) and FP64-level accuracy.  Writes Un of s as double-float
+// words: the FP64 conversions run on the FP64 pipe too.
 template <class C>
-__device__ __forceinline__ void near_row_dd(const FusedArgs<C>& a, int s, int lane) {
+__device__ __noinline__ void near_row_dd(const FusedArgs<C>& a, int s, int lane) {
   const longlong2 mt = __ldg(a.nr_meta + s);
   const int64_t r = mt.x;
   const int j0 = (int)(mt.y >> 32), ns = (int)(mt.y & 0xffffffffll);
-  const cplxf* qh = a.nc_hi + r;
-  const cplxf* ql = a.nc_lo + r;
-  const cplxf* dh = a.dens_dd;
-  const cplxf* dl = a.dens_dd + 2 * a.E;
+  // a block's four hi (lo) parts are 32 bytes, a source's two hi (lo) densities 16:
+  // 16-byte loads; the next pass's source index is fetched ahead
+  const float4* qh = reinterpret_cast<const float4*>(a.nc_hi + r);
+  const float4* ql = reinterpret_cast<const float4*>(a.nc_lo + r);
+  const float4* dh = reinterpret_cast<const float4*>(a.dens_dd);
+  const float4* dl = reinterpret_cast<const float4*>(a.dens_dd + 2 * a.E);
   const int* src = a.nc_src + j0;
   dflt ur{0, 0}, ui{0, 0}, dr{0, 0}, di{0, 0};
+  int f = lane < ns ? __ldg(src + lane) : 0;
+#pragma unroll 1
   for (int j = lane; j < ns; j += 32) {
-    const int f = src[j];
-    const cplxf ph = ldcg(dh + 2 * f), pl = ldcg(dl + 2 * f), vh = ldcg(dh + 2 * f + 1), vl = ldcg(dl + 2 * f + 1);
-    dd_cmac(ur, ui, qh[4 * j], ql[4 * j], ph, pl);
-    dd_cmac(ur, ui, qh[4 * j + 1], ql[4 * j + 1], vh, vl);
-    dd_cmac(dr, di, qh[4 * j + 2], ql[4 * j + 2], ph, pl);
-    dd_cmac(dr, di, qh[4 * j + 3], ql[4 * j + 3], vh, vl);
+    const float4 h = __ldcg(dh + f), l = __ldcg(dl + f);
+    const float4 h0 = __ldg(qh + 2 * j), h1 = __ldg(qh + 2 * j + 1), l0 = __ldg(ql + 2 * j), l1 = __ldg(ql + 2 * j + 1);
+    f = j + 32 < ns ? __ldg(src + j + 32) : 0;
+    const cplxf ph{h.x, h.y}, pl{l.x, l.y}, vh{h.z, h.w}, vl{l.z, l.w};
+    dd_cmac(ur, ui, cplxf{h0.x, h0.y}, cplxf{l0.x, l0.y}, ph, pl);
+    dd_cmac(dr, di, cplxf{h1.x, h1.y}, cplxf{l1.x, l1.y}, ph, pl);
+    dd_cmac(ur, ui, cplxf{h0.z, h0.w}, cplxf{l0.z, l0.w}, vh, vl);
+    dd_cmac(dr, di, cplxf{h1.z, h1.w}, cplxf{l1.z, l1.w}, vh, vl);
   }
-  ur = dd_wsum(ur);
-  ui = dd_wsum(ui);
-  dr = dd_wsum(dr);
-  di = dd_wsum(di);
-  if (lane == 0) {
-    reinterpret_cast<cplx*>(a.Un)[2 * s] = cplx{dd_value(ur), dd_value(ui)};
-    reinterpret_cast<cplx*>(a.Un)[2 * s + 1] = cplx{dd_value(dr), dd_value(di)};
+  const dflt v = dd_wsum4(ur, ui, dr, di, lane);
+  if ((lane & 7) == 0) {
+    float* o = reinterpret_cast<float*>(a.Un) + 8 * (size_t)s + 4 * (lane >> 4) + ((lane >> 3) & 1);
+    o[0] = v.h;
+    o[2] = v.l;
   }
 }
 
@@ -727,7 +783,7 @@ __device__ __forceinline__ void near_row_diff(const FusedArgs<cplxf>& a, int s, 
 
 template <class C>
 __device__ __forceinline__ void near_row(const FusedArgs<C>& a, int s, int lane) {
-  if (a.nc_lo) {
+  if (sizeof(C) == sizeof(cplx) && a.nc_lo) {
     near_row_dd(a, s, lane);
     return;
   }
@@ -1756,6 +1812,54 @@ __device__ bool tc_m2l_item(const FusedArgs<cplxf>& a, int l, int item, unsigned
   return true;
 }
 
+// Asks the L2 for `bytes` from p on, a line per thread of the G blocks: the tables of
+// the next stage, which the near-field stream (more than the L2 holds in the FP64
+// product) has pushed out since the last product; every load of a stage that misses
+// would wait for DRAM in a chain of a few such batches.
+__device__ __forceinline__ void l2_prefetch(const void* p, size_t bytes, int bid, int G) {
+  const char* c = static_cast<const char*>(p);
+  for (size_t o = ((size_t)bid * nt() + threadIdx.x) * 128; o < bytes; o += (size_t)G * nt() * 128)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(c + o));
+}
+// The tables of the M2M into level l, of the M2L and L2L into level l, of L2P.
+template <class C>
+__device__ __forceinline__ void prefetch_m2m(const FusedArgs<C>& a, int l, int bid, int G) {
+  const size_t n = (size_t)4 * a.S[l + 1] * a.S[l] * sizeof(cplxf);
+  if (sizeof(C) == sizeof(cplx) && a.m2ml[l]) {
+    l2_prefetch(a.m2mh[l], n, bid, G);
+    l2_prefetch(a.m2ml[l], n, bid, G);
+  } else {
+    l2_prefetch(a.m2m[l], n / sizeof(cplxf) * sizeof(C), bid, G);
+  }
+}
+template <class C>
+__device__ __forceinline__ void prefetch_down(const FusedArgs<C>& a, int l, int bid, int G) {
+  const size_t n = (size_t)49 * a.S[l] * a.S[l] * sizeof(cplxf), nl = (size_t)4 * a.S[l - 1] * a.S[l] * sizeof(cplxf);
+  if (sizeof(C) == sizeof(cplx) && a.m2ltl[l]) {
+    l2_prefetch(a.m2lth[l], n, bid, G);
+    l2_prefetch(a.m2ltl[l], n, bid, G);
+    if (a.l2ll[l - 1]) {
+      l2_prefetch(a.l2lh[l - 1], nl, bid, G);
+      l2_prefetch(a.l2ll[l - 1], nl, bid, G);
+    }
+  } else if (sizeof(C) == sizeof(cplxf)) {
+    l2_prefetch(a.m2lt[l], n, bid, G);
+    l2_prefetch(a.l2l[l - 1], nl, bid, G);
+  }
+}
+template <class C>
+__device__ __forceinline__ void prefetch_l2p(const FusedArgs<C>& a, int bid, int G) {
+  const size_t n = (size_t)2 * a.P[a.D] * a.E * sizeof(cplxf);
+  if (sizeof(C) == sizeof(cplx) && a.l2pl) {
+    l2_prefetch(a.l2ph, n, bid, G);
+    l2_prefetch(a.l2pl, n, bid, G);
+  } else if (sizeof(C) == sizeof(cplxf)) {
+    const int O = a.O[a.D];
+    l2_prefetch(a.l2p + (size_t)O * a.E, n / 2, bid, G);
+    l2_prefetch(a.l2p + (size_t)(a.S[a.D] + O) * a.E, n / 2, bid, G);
+  }
+}
+
 // Block items of the next stage, so that a block can stage their operators in
 // shared memory at the end of the current stage (off the next stage's critical
 // path): the M2M quadrant stack of a B stage, the first M2L chunk's operator and
@@ -1768,6 +1872,19 @@ __device__ __forceinline__ bool bstage_quad(const FusedArgs<C>& a, int l, int ws
   *ng = quad ? (a.nne[l] + nw() - 1) / nw() : 0;
   return quad;
 }
+// FP64 product in double-float arithmetic, levels whose pairs are few: M2L items of
+// one warp per (pair, 32 targets, share of the sources), the operator rows read from
+// L2; the number of shares (up to four), or 0 for staged chunks.  A chunk's chain is
+// its operator's copy and two whole translations per warp, about 20 us however few
+// its pairs; the direct items of up to one and a half rounds of the
+// grid's warps 12 to 30 (2416 pairs of level 4 of the 8x8 hexagon block: 51 against 30).
+template <class C>
+__device__ __forceinline__ int m2l_direct(const FusedArgs<C>& a, int l, int wstride) {
+  if (sizeof(C) != sizeof(cplx) || !a.m2ltl[l] || a.P[l] > PF_NCOEF) return 0;
+  const int n = a.npair[l] * ((a.P[l] + 31) >> 5);
+  if (n == 0 || 2 * n > 3 * wstride) return a.P[l] > TSP ? 1 : 0;
+  return max(1, min(4, wstride / n));
+}
 struct DItems {
   bool ql2l;
   int ntc, nchu, ngl, nl2l;
@@ -1778,7 +1895,7 @@ __device__ __forceinline__ DItems dstage_items(const FusedArgs<C>& a, int l, int
   const bool top = (int64_t)a.nne[l] * P <= wstride;
   DItems d;
   d.nl2l = top ? a.nne[l] * P : a.nne[l];
-  const bool wpair = a.m2l_warp || P > TSP;
+  const bool wpair = a.m2l_warp || P > TSP || m2l_direct(a, l, wstride) > 0;
   d.ql2l = sizeof(C) == sizeof(cplxf) && !top && Pp <= PF_NCOEF && 4 * Pp * P <= (a.tregL > 0 ? a.tregL : a.treg);
   const bool tcl = TC && sizeof(C) == sizeof(cplxf) && a.tc_kp[l] > 0;
   d.ntc = tcl ? a.tc_ntile[l] * a.tc_ngrp[l] : 0;
@@ -1790,7 +1907,19 @@ __device__ __forceinline__ DItems dstage_items(const FusedArgs<C>& a, int l, int
 template <class C>
 __device__ __forceinline__ void stage_chunk(const FusedArgs<C>& a, int l, int b, C* sT) {
   const int P = a.P[l], S = a.S[l], O = a.O[l];
-  const C* To = a.m2lt[l] + (size_t)a.ch_off[l][b] * S * S + (size_t)O * S + O;   // [n source][l target]
+  const size_t ob = (size_t)a.ch_off[l][b] * S * S + (size_t)O * S + O;           // [n source][l target]
+  if (sizeof(C) == sizeof(cplx) && a.m2ltl[l]) {
+    // double-float words [source][target] (S = P in the FP64 product), eight loads in flight
+    float4* w = reinterpret_cast<float4*>(sT);
+    const cplxf *Th = a.m2lth[l] + ob, *Tl = a.m2ltl[l] + ob;
+#pragma unroll 4
+    for (int t = threadIdx.x; t < P * P; t += nt()) {
+      const cplxf h = Th[t], lo = Tl[t];
+      w[t] = make_float4(h.re, h.im, lo.re, lo.im);
+    }
+    return;
+  }
+  const C* To = a.m2lt[l] + ob;
   if (S == P)
     stage_copy(sT, To, P * P, IdxTranspose{P});
   else
@@ -1801,75 +1930,160 @@ __device__ __forceinline__ void stage_l2l_quad(const FusedArgs<C>& a, int l, C* 
   stage_copy_quad(dst, a.l2l[l - 1] + (size_t)a.O[l - 1] * a.S[l] + a.O[l], a.P[l], a.P[l - 1], a.S[l], a.S[l - 1]);
 }
 
+// M2M into the nbi boxes of level l in double-float arithmetic (FP64 product), a box per
+// block: the warps share its four quadrants and the two halves of its (at most 64)
+// coefficients, each reads its operator rows from L2 and the quadrants' sums meet in
+// shared memory.  Bound by the loads' latency, one chain of Pc / 7 batches; with the
+// operators staged quadrant after quadrant (a box per warp) the same level took four
+// copies and four chains: 42 against
+// 17 us on the level-5 boxes of the 8x8 hexagon block.
+template <class C>
+__device__ void m2m_split_dd(const FusedArgs<C>& a, int l, int nbi, unsigned char* sm, int warp, int lane, int rb,
+                             int G) {
+  if (rb >= nbi) return;
+  const int P = a.P[l], Pc = a.P[l + 1], S = a.S[l], O = a.O[l], Sc = a.S[l + 1], Oc = a.O[l + 1];
+  float4* w = reinterpret_cast<float4*>(sm);               // [4 Pc]
+  float4* red = w + PF_NCOEF;                              // [4][64] (re.h, re.l, im.h, im.l)
+  const int q = warp & 3, n = lane + 32 * (warp >> 2);
+  for (int i = rb; i < nbi; i += G) {
+    const int box = a.ne[l][i];
+    __syncthreads();
+    for (int t = threadIdx.x; t < 4 * Pc; t += nt()) {
+      const int c = t / Pc, ch = 4 * box + c;
+      const bool on = a.bb[l + 1][ch] < a.be[l + 1][ch];
+      w[t] = on ? __ldcg(a.Mw[l + 1] + (size_t)ch * Sc + Oc + (t - c * Pc)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    dflt re{0, 0}, im{0, 0};
+    if (n < P && a.bb[l + 1][4 * box + q] < a.be[l + 1][4 * box + q]) {
+      const size_t o = (size_t)(q * Sc + Oc) * S + O + n;
+      dd_rows(re, im, a.m2mh[l] + o, a.m2ml[l] + o, S, w + q * Pc, Pc);
+    }
+    red[q * 64 + n] = make_float4(re.h, re.l, im.h, im.l);
+    __syncthreads();
+    if (threadIdx.x < P) {
+      dflt r{0, 0}, m{0, 0};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float4 v = red[c * 64 + threadIdx.x];
+        r = dd_add(r, dflt{v.x, v.y});
+        m = dd_add(m, dflt{v.z, v.w});
+      }
+      a.M[l][(size_t)box * S + O + threadIdx.x] = from_d<C>(cplx{dd_value(r), dd_value(m)});
+      a.Mw[l][(size_t)box * S + O + threadIdx.x] = dd_word(r, m);
+    }
+  }
+  __syncthreads();
+}
+
+// M2L of a chunk's pairs pb .. pe (at most two per warp, one offset) in double-float
+// arithmetic (FP64 product), the operator staged as 16-byte words [source][target].
+// The lanes take the outputs 0 .. 31 of both pairs together (one operator word for two
+// products), then outputs 32 .. 47 of one pair on each half warp, then what is left
+// of P <= 49 with the lanes over the sources.
+template <class C>
+__device__ __forceinline__ void m2l_chunk_dd(const FusedArgs<C>& a, int l, int pb, int pe, const float4* T, C* wsm,
+                                             int warp, int lane) {
+  const int P = a.P[l], S = a.S[l], O = a.O[l];
+  float4* w = reinterpret_cast<float4*>(wsm);              // [2][P]
+  for (int pi = pb + 2 * warp; pi < pe; pi += 2 * nw()) {
+    const bool two = pi + 1 < pe;
+    const int pj = two ? pi + 1 : pi;
+    const int srcA = a.pr_src[l][pi], srcB = a.pr_src[l][pj];
+    const int mA = a.pr_img[l][pi], mB = a.pr_img[l][pj];
+    C* LA = a.L[l] + (size_t)a.pr_tgt[l][pi] * S + O;
+    C* LB = a.L[l] + (size_t)a.pr_tgt[l][pj] * S + O;
+    __syncwarp();
+    for (int m = lane; m < P; m += 32) {
+      w[m] = dd_phase(a.alpha_w, mA, __ldcg(a.Mw[l] + (size_t)srcA * S + O + m));
+      if (two) w[P + m] = dd_phase(a.alpha_w, mB, __ldcg(a.Mw[l] + (size_t)srcB * S + O + m));
+    }
+    __syncwarp();
+    auto put = [&](C* L, int n, dflt re, dflt im) { atomic_add(L + n, from_d<C>(cplx{dd_value(re), dd_value(im)})); };
+    if (lane < P) {
+      dflt r0{0, 0}, i0{0, 0}, r1{0, 0}, i1{0, 0};
+      if (two) {
+#pragma unroll 2
+        for (int m = 0; m < P; ++m) {
+          const float4 t = T[m * P + lane];
+          dd_cmac(r0, i0, t, w[m]);
+          dd_cmac(r1, i1, t, w[P + m]);
+        }
+        put(LB, lane, r1, i1);
+      } else {
+#pragma unroll 2
+        for (int m = 0; m < P; ++m) dd_cmac(r0, i0, T[m * P + lane], w[m]);
+      }
+      put(LA, lane, r0, i0);
+    }
+    if (P > 32) {
+      const int h = lane >> 4, n = 32 + (lane & 15);
+      if (n < P && (h == 0 || two)) {
+        dflt re{0, 0}, im{0, 0};
+        const float4* wh = w + h * P;
+#pragma unroll 2
+        for (int m = 0; m < P; ++m) dd_cmac(re, im, T[m * P + n], wh[m]);
+        put(h ? LB : LA, n, re, im);
+      }
+      for (int e = 48; e < P; ++e) {
+        dflt re{0, 0}, im{0, 0};
+        if (h == 0 || two)
+          for (int m = lane & 15; m < P; m += 16) dd_cmac(re, im, T[m * P + e], w[h * P + m]);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+          re = dd_add(re, dflt{__shfl_down_sync(0xffffffffu, re.h, o, 16), __shfl_down_sync(0xffffffffu, re.l, o, 16)});
+          im = dd_add(im, dflt{__shfl_down_sync(0xffffffffu, im.h, o, 16), __shfl_down_sync(0xffffffffu, im.l, o, 16)});
+        }
+        if ((lane & 15) == 0 && (h == 0 || two)) put(h ? LB : LA, e, re, im);
+      }
+    }
+  }
+}
+
 template <class C>
 __device__ void m2m_staged(const FusedArgs<C>& a, int l, int nbi, int wfirst, int wstride, C* sT, C* wsm, int lane,
                            int bid) {
   const int P = a.P[l], Pc = a.P[l + 1], PP = Pc * P;
   const int S = a.S[l], O = a.O[l], Sc = a.S[l + 1], Oc = a.O[l + 1];
-  const bool dd = a.m2ml[l] != nullptr;
   const int rounds = (nbi + wstride - 1) / wstride;
   for (int rd = 0; rd < rounds; ++rd) {
     if (bid + rd * wstride >= nbi) break;
     const int i = wfirst + rd * wstride;
     const bool mine = i < nbi;
     const int box = mine ? a.ne[l][i] : 0;
-    cplxf* wh = reinterpret_cast<cplxf*>(wsm);
-    cplxf* wl = wh + PF_NCOEF;
     __syncwarp();
     if (mine) {
       for (int t = lane; t < 4 * Pc; t += 32) {
         const int q = t / Pc, ch = 4 * box + q;
-        const C v = a.bb[l + 1][ch] < a.be[l + 1][ch] ? ldcg(a.M[l + 1] + (size_t)ch * Sc + Oc + (t - q * Pc))
-                                                      : C{0, 0};
-        if (dd) {
-          const cplx d = to_d(v);
-          wh[t] = cplxf{(float)d.re, (float)d.im};
-          wl[t] = split_lo(d);
-        } else {
-          wsm[t] = v;
-        }
+        wsm[t] = a.bb[l + 1][ch] < a.be[l + 1][ch] ? ldcg(a.M[l + 1] + (size_t)ch * Sc + Oc + (t - q * Pc)) : C{0, 0};
       }
     }
     C acc[2] = {C{0, 0}, C{0, 0}};
-    dflt re[2] = {{0, 0}, {0, 0}}, im[2] = {{0, 0}, {0, 0}};
     for (int q = 0; q < 4; ++q) {
       __syncthreads();
       // the used [Pc][P] block of T_q: source rows q Sc + Oc + m, target columns O + n
-      if (dd) {
-        cplxf* th = reinterpret_cast<cplxf*>(sT);
-        stage_copy(th, a.m2mh[l] + (size_t)(q * Sc + Oc) * S + O, PP, IdxBlock{P, S});
-        stage_copy(th + PP, a.m2ml[l] + (size_t)(q * Sc + Oc) * S + O, PP, IdxBlock{P, S});
-      } else {
-        stage_copy(sT, a.m2m[l] + (size_t)(q * Sc + Oc) * S + O, PP, IdxBlock{P, S});
-      }
+      stage_copy(sT, a.m2m[l] + (size_t)(q * Sc + Oc) * S + O, PP, IdxBlock{P, S});
       __syncthreads();
       if (!mine) continue;
       for (int h = 0; h < 2; ++h) {
         const int n = lane + 32 * h;
         if (n >= P) break;
-        if (dd) {
-          const cplxf* th = reinterpret_cast<const cplxf*>(sT);
+        C s0{0, 0}, s1{0, 0};
+        int m = 0;
 #pragma unroll 4
-          for (int m = 0; m < Pc; ++m)
-            dd_cmac(re[h], im[h], th[m * P + n], th[PP + m * P + n], wh[q * Pc + m], wl[q * Pc + m]);
-        } else {
-          C s0{0, 0}, s1{0, 0};
-          int m = 0;
-#pragma unroll 4
-          for (; m + 1 < Pc; m += 2) {
-            s0 += sT[m * P + n] * wsm[q * Pc + m];
-            s1 += sT[(m + 1) * P + n] * wsm[q * Pc + m + 1];
-          }
-          if (m < Pc) s0 += sT[m * P + n] * wsm[q * Pc + m];
-          acc[h] += s0 + s1;
+        for (; m + 1 < Pc; m += 2) {
+          s0 += sT[m * P + n] * wsm[q * Pc + m];
+          s1 += sT[(m + 1) * P + n] * wsm[q * Pc + m + 1];
         }
+        if (m < Pc) s0 += sT[m * P + n] * wsm[q * Pc + m];
+        acc[h] += s0 + s1;
       }
     }
     if (mine) {
       for (int h = 0; h < 2; ++h) {
         const int n = lane + 32 * h;
         if (n >= P) break;
-        a.M[l][(size_t)box * S + O + n] = dd ? from_d<C>(cplx{dd_value(re[h]), dd_value(im[h])}) : acc[h];
+        a.M[l][(size_t)box * S + O + n] = acc[h];
       }
     }
   }
@@ -1884,11 +2098,7 @@ __device__ void l2l_staged(const FusedArgs<C>& a, int l, int nl2l, int wfirst, i
                            int bid) {
   const int P = a.P[l], Pp = a.P[l - 1], PP = Pp * P;
   const int S = a.S[l], O = a.O[l], Sp = a.S[l - 1], Op = a.O[l - 1];
-  // FP64 product: double-float arithmetic from the hi and lo tables
-  const bool dd = a.l2ll[l - 1] != nullptr;
   const int rounds = (nl2l + wstride - 1) / wstride;
-  cplxf* wh = reinterpret_cast<cplxf*>(wsm);
-  cplxf* wl = wh + PF_NCOEF;
   for (int rd = 0; rd < rounds; ++rd) {
     if (bid + rd * wstride >= nl2l) break;
     const int i = wfirst + rd * wstride;
@@ -1896,37 +2106,14 @@ __device__ void l2l_staged(const FusedArgs<C>& a, int l, int nl2l, int wfirst, i
     const int box = mine ? a.ne[l][i] : 0, par = box >> 2, qb = box & 3;
     __syncwarp();
     if (mine)
-      for (int m = lane; m < Pp; m += 32) {
-        const C v = ldcg(a.L[l - 1] + (size_t)par * Sp + Op + m);
-        if (dd) {
-          const cplx d = to_d(v);
-          wh[m] = cplxf{(float)d.re, (float)d.im};
-          wl[m] = split_lo(d);
-        } else {
-          wsm[m] = v;
-        }
-      }
+      for (int m = lane; m < Pp; m += 32) wsm[m] = ldcg(a.L[l - 1] + (size_t)par * Sp + Op + m);
     for (int q = 0; q < 4; ++q) {
       __syncthreads();
       // the used [Pp][P] block of T_q: source rows q Sp + Op + m, target columns O + n
-      if (dd) {
-        cplxf* th = reinterpret_cast<cplxf*>(sT);
-        stage_copy(th, a.l2lh[l - 1] + (size_t)(q * Sp + Op) * S + O, PP, IdxBlock{P, S});
-        stage_copy(th + PP, a.l2ll[l - 1] + (size_t)(q * Sp + Op) * S + O, PP, IdxBlock{P, S});
-      } else {
-        stage_copy(sT, a.l2l[l - 1] + (size_t)(q * Sp + Op) * S + O, PP, IdxBlock{P, S});
-      }
+      stage_copy(sT, a.l2l[l - 1] + (size_t)(q * Sp + Op) * S + O, PP, IdxBlock{P, S});
       __syncthreads();
       if (!mine || qb != q) continue;
       for (int n = lane; n < P; n += 32) {
-        if (dd) {
-          const cplxf* th = reinterpret_cast<const cplxf*>(sT);
-          dflt re{0, 0}, im{0, 0};
-#pragma unroll 4
-          for (int m = 0; m < Pp; ++m) dd_cmac(re, im, th[m * P + n], th[PP + m * P + n], wh[m], wl[m]);
-          atomic_add(a.L[l] + (size_t)box * S + O + n, from_d<C>(cplx{dd_value(re), dd_value(im)}));
-          continue;
-        }
         C s0{0, 0}, s1{0, 0};
         int m = 0;
 #pragma unroll 4
@@ -1949,6 +2136,7 @@ __device__ void l2l_staged(const FusedArgs<C>& a, int l, int nl2l, int wfirst, i
 template <class C, bool TC>
 __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid, const int G) {
   extern __shared__ __align__(128) unsigned char smraw[];
+  constexpr bool F64 = sizeof(C) == sizeof(cplx);
   C* sm = reinterpret_cast<C*>(smraw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wfirst = warp_first(bid, warp, G), wstride = G * nw();
@@ -2036,6 +2224,10 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
 
   // ------------------------------------------------------------ A: gather + P2M, clear L; fiber part
   {
+    if (D - 1 >= (a.top3 ? 2 : 0))
+      prefetch_m2m(a, D - 1, bid, G);
+    else
+      prefetch_down(a, 1, bid, G);
     for (int l = 1; l <= D; ++l) {
       C* Lz = a.L[l];
       const size_t nz = (size_t)a.nbox[l] * a.S[l];
@@ -2048,7 +2240,56 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
     const int gA = G - a.fblk;
     if (bid < gA) {
       const int PD = a.P[D];
-      for (int i = warp_first(bid, warp, gA); i < a.nne[D]; i += gA * nw()) {
+      if (F64 && a.p2ml) {
+        // FP64 product in double-float arithmetic: one warp per leaf and 32
+        // coefficients; the warp gathers 32 elements at a time into its shared
+        // memory (the first 32 coefficients' warp also writes the densities).  A leaf per warp, one element
+        // after another, was the stage's longest chain (60 us on a 64-element leaf).
+        float4* w = reinterpret_cast<float4*>(wsm);            // [32][2]
+        const int NH = (PD + 31) >> 5;
+        for (int i = warp_first(bid, warp, gA); i < a.nne[D] * NH; i += gA * nw()) {
+          const int box = a.ne[D][i / NH], hp = i % NH, s0 = a.bb[D][box], s1 = a.be[D][box];
+          const int n = 32 * hp + lane;
+          dflt re{0, 0}, im{0, 0};
+          for (int sb = s0; sb < s1; sb += 32) {
+            const int s = sb + lane;
+            __syncwarp();
+            if (s < s1) {
+              const int ei = a.perm[s];
+              const cplx p = a.ph[s];
+              const cplx e0 = p * a.x[2 * ei], e1 = p * a.x[2 * ei + 1];
+              const float4 d0 = dd_word(e0), d1 = dd_word(e1);
+              w[2 * lane] = d0;
+              w[2 * lane + 1] = d1;
+              if (hp == 0) {
+                a.dens[2 * s] = from_d<C>(e0);
+                a.dens[2 * s + 1] = from_d<C>(e1);
+                float4* dh = reinterpret_cast<float4*>(a.dens_dd);
+                dh[s] = make_float4(d0.x, d0.y, d1.x, d1.y);
+                dh[a.E + s] = make_float4(d0.z, d0.w, d1.z, d1.w);
+              }
+            }
+            __syncwarp();
+            if (n < PD) {
+              const int cnt = min(32, s1 - sb);
+              const size_t c = (size_t)sb * 2 * PD + n;
+              const cplxf *ch = a.p2mh + c, *cl = a.p2ml + c;
+#pragma unroll 4
+              for (int f = 0; f < cnt; ++f) {
+                const float4 d0 = w[2 * f], d1 = w[2 * f + 1];
+                const size_t k0 = (size_t)f * 2 * PD, k1 = k0 + PD;
+                dd_cmac(re, im, ch[k0], cl[k0], cplxf{d0.x, d0.y}, cplxf{d0.z, d0.w});
+                dd_cmac(re, im, ch[k1], cl[k1], cplxf{d1.x, d1.y}, cplxf{d1.z, d1.w});
+              }
+            }
+          }
+          if (n < PD) {
+            a.M[D][(size_t)box * PD + n] = from_d<C>(cplx{dd_value(re), dd_value(im)});
+            a.Mw[D][(size_t)box * PD + n] = dd_word(re, im);
+          }
+        }
+      }
+      for (int i = warp_first(bid, warp, gA); !(F64 && a.p2ml) && i < a.nne[D]; i += gA * nw()) {
         const int box = a.ne[D][i], s0 = a.bb[D][box], s1 = a.be[D][box];
         // the leaf's elements GU x 32 at a time: indices and phases, then the
         // inputs, each batch of loads issued before its first use
@@ -2075,12 +2316,6 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
             const cplx e0 = p * xa[k], e1 = p * xb[k];     // FP64, then rounded
             a.dens[2 * s] = from_d<C>(e0);
             a.dens[2 * s + 1] = from_d<C>(e1);
-            if (a.dens_dd) {
-              a.dens_dd[2 * s] = cplxf{(float)e0.re, (float)e0.im};
-              a.dens_dd[2 * s + 1] = cplxf{(float)e1.re, (float)e1.im};
-              a.dens_dd[2 * a.E + 2 * s] = split_lo(e0);
-              a.dens_dd[2 * a.E + 2 * s + 1] = split_lo(e1);
-            }
             if (a.dlo) {
               a.dlo[2 * s] = split_lo(e0);
               a.dlo[2 * s + 1] = split_lo(e1);
@@ -2089,22 +2324,6 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
           }
         }
         __syncwarp();
-        if (a.p2ml) {
-          // FP64 product in double-float arithmetic, from the densities' hi and
-          // lo parts just written by this warp
-          const cplxf* dh = a.dens_dd;
-          const cplxf* dl = a.dens_dd + 2 * a.E;
-          for (int n = lane; n < PD; n += 32) {
-            dflt re{0, 0}, im{0, 0};
-            for (int f = s0; f < s1; ++f) {
-              const size_t c0 = (size_t)f * 2 * PD + n, c1 = c0 + PD;
-              dd_cmac(re, im, a.p2mh[c0], a.p2ml[c0], dh[2 * f], dl[2 * f]);
-              dd_cmac(re, im, a.p2mh[c1], a.p2ml[c1], dh[2 * f + 1], dl[2 * f + 1]);
-            }
-            a.M[D][(size_t)box * PD + n] = from_d<C>(cplx{dd_value(re), dd_value(im)});
-          }
-          continue;
-        }
         const int SD = a.S[D], OD = a.O[D];
         // coefficients n < 32 (PD & ~31) a lane each over all the leaf's
         // elements; the last PD mod 32 split over lane groups that share the
@@ -2174,12 +2393,18 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
   for (int l = D - 1; l >= lstop; --l) {
     const int P = a.P[l], Pc = a.P[l + 1];
     const int jst = D - 1 - l;
+    if (l - 1 >= lstop)
+      prefetch_m2m(a, l - 1, bid, G);
+    else
+      prefetch_down(a, 1, bid, G);
     const int r0 = a.near_first ? (jst == 0 ? 0 : NI) : (int)((int64_t)NI * jst / nst);
     const int r1 = a.near_first ? NI : (int)((int64_t)NI * (jst + 1) / nst);
     // near the top of the tree the boxes are too few to occupy the grid: one
     // warp per output coefficient, lanes over the 4 Pc child coefficients.  The
     // root then forms L(0) = (R T_0) [M(1) of its four children] at once.
     const bool top = (int64_t)a.nne[l] * P <= wstride;
+    // FP64 product in double-float arithmetic: a box per block
+    const bool split = F64 && !top && l >= 1 && a.m2ml[l] && P <= 64 && 4 * Pc <= PF_NCOEF && nw() == 8;
     const int nbi = top ? a.nne[l] * P : a.nne[l];
     // with top3, the level-2 stage adds M(1) (one warp per coefficient, from the
     // 16 level-3 boxes below)
@@ -2189,8 +2414,10 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
     // shared memory once and applies it to all of its warps' boxes (a warp on
     // its own would stream the whole [4][Pc][P] table from L2 for every box)
     const bool quad = sizeof(C) == sizeof(cplxf) && l >= 1 && !top && 4 * Pc <= PF_NCOEF && 4 * Pc * P <= a.treg;
-    const bool staged = quad || (l >= 1 && !top && 4 * Pc <= PF_NCOEF && Pc * P <= TSIZE && P <= 64);
-    if (quad) {
+    const bool staged = split || quad || (l >= 1 && !top && 4 * Pc <= PF_NCOEF && Pc * P <= TSIZE && P <= 64);
+    if (split) {
+      m2m_split_dd(a, l, nbi, smraw, warp, lane, rank(ks - 1), G);
+    } else if (quad) {
       m2m_quad(a, l, nbi, sT, wsm, warp, lane, rank(ks - 1), pf_b == l,
                a.bdone ? a.bdone + (size_t)(ks - 1) * G + bid : nullptr, G);
       pf_b = -1;
@@ -2217,7 +2444,10 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
           acc += A[v] * ldcg(M3 + v);
         }
         acc = wsum(acc);
-        if (lane == 0) a.M[1][(size_t)b1 * a.S[1] + a.O[1] + n] = acc;
+        if (lane == 0) {
+          a.M[1][(size_t)b1 * a.S[1] + a.O[1] + n] = acc;
+          if (F64 && a.Mw[1]) a.Mw[1][(size_t)b1 * a.S[1] + a.O[1] + n] = dd_word(to_d(acc));
+        }
         continue;
       }
       if (top) {
@@ -2249,30 +2479,27 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
             a.L[0][(size_t)box * S + a.O[0] + n] = acc;
           else
             a.M[l][(size_t)box * S + a.O[l] + n] = acc;
+          if (F64 && l > 0 && a.Mw[l]) a.Mw[l][(size_t)box * S + a.O[l] + n] = dd_word(to_d(acc));
         }
         continue;
       }
       const int box = a.ne[l][i];
-      if (a.m2ml[l] && 4 * Pc <= PF_NCOEF) {
+      if (F64 && a.m2ml[l] && 4 * Pc <= PF_NCOEF) {   // orders above 64 coefficients
         // FP64 product in double-float arithmetic: the four children's
         // multipoles split into hi and lo parts, the operator from its tables
-        cplxf* wh = reinterpret_cast<cplxf*>(wsm);
-        cplxf* wl = wh + PF_NCOEF;
+        float4* w = reinterpret_cast<float4*>(wsm);
         __syncwarp();
         for (int t = lane; t < 4 * Pc; t += 32) {
           const int q = t / Pc, ch = 4 * box + q;
-          const cplx v = a.bb[l + 1][ch] < a.be[l + 1][ch] ? to_d(ldcg(a.M[l + 1] + (size_t)ch * Pc + (t - q * Pc)))
-                                                           : cplx{0, 0};
-          wh[t] = cplxf{(float)v.re, (float)v.im};
-          wl[t] = split_lo(v);
+          w[t] = a.bb[l + 1][ch] < a.be[l + 1][ch] ? __ldcg(a.Mw[l + 1] + (size_t)ch * Pc + (t - q * Pc))
+                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         __syncwarp();
         for (int n = lane; n < P; n += 32) {
           dflt re{0, 0}, im{0, 0};
-#pragma unroll 4
-          for (int u = 0; u < 4 * Pc; ++u)
-            dd_cmac(re, im, a.m2mh[l][(size_t)u * P + n], a.m2ml[l][(size_t)u * P + n], wh[u], wl[u]);
+          dd_rows(re, im, a.m2mh[l] + n, a.m2ml[l] + n, P, w, 4 * Pc);
           a.M[l][(size_t)box * P + n] = from_d<C>(cplx{dd_value(re), dd_value(im)});
+          if (l > 0) a.Mw[l][(size_t)box * P + n] = dd_word(re, im);
         }
       } else {
         // the generic form (the FP32 product may run at orders below its
@@ -2290,7 +2517,10 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
             __syncwarp();
             if (n < P) acc += colmv(a.m2m[l] + (size_t)(q * Sc + Oc) * S + O + n, S, wsm, Pc);
           }
-          if (n < P) a.M[l][(size_t)box * S + O + n] = acc;
+          if (n < P) {
+            a.M[l][(size_t)box * S + O + n] = acc;
+            if (F64 && l > 0 && a.Mw[l]) a.Mw[l][(size_t)box * S + O + n] = dd_word(to_d(acc));
+          }
         }
       }
       if (l == 0) {
@@ -2324,13 +2554,21 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
   // ------------------------------------------------------------ D: L2L + M2L
   for (int l = 1; l <= D; ++l) {
     const int P = a.P[l], Pp = a.P[l - 1];
+    if (l < D)
+      prefetch_down(a, l + 1, bid, G);
+    else
+      prefetch_l2p(a, bid, G);
     // L2L: one warp per output coefficient while the boxes are few, else one
     // warp per box
     const bool top = (int64_t)a.nne[l] * P <= wstride;
-    const int nl2l = top ? a.nne[l] * P : a.nne[l];
+    // (FP64 product in double-float arithmetic: one warp per box and 32 coefficients)
+    const bool dl2l = F64 && !top && a.l2ll[l - 1] && Pp <= PF_NCOEF;
+    const int NH = (P + 31) >> 5;
+    const int nl2l = top ? a.nne[l] * P : dl2l ? a.nne[l] * NH : a.nne[l];
     // M2L one warp per pair (operator rows through L1/L2), or one block per
     // chunk of pairs sharing the offset (operator staged in shared memory)
-    const bool wpair = a.m2l_warp || P > TSP;
+    const int ksh = m2l_direct(a, l, wstride);
+    const bool wpair = a.m2l_warp || P > TSP || ksh > 0;
     // L2L as block items (groups of nw() boxes, the stacked quadrant operators
     // staged once per block) when the FP32 tables fit the staging region
     // M2L on the tensor cores at this level (FP32 product): block items over
@@ -2368,6 +2606,10 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
         __syncthreads();                                      // sT of the previous chunk is done
         if (!(b0 == rb && pf_c == b && pf_cl == l)) stage_chunk(a, l, b, sT);
         __syncthreads();
+        if (F64 && a.m2ltl[l]) {
+          m2l_chunk_dd(a, l, pb, pe, reinterpret_cast<const float4*>(sT), wsm, warp, lane);
+          continue;
+        }
         // two pairs per warp pass, sharing the operator rows read from shared memory
         for (int pi = pb + 2 * warp; pi < pe; pi += 2 * nw()) {
           const bool two = pi + 1 < pe;
@@ -2393,9 +2635,9 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
     if (a.bdone && threadIdx.x == 0) a.bdone[(size_t)(ks - 1) * G + bid] = gtimer();
     // box-form L2L with the quadrant operators staged in shared memory, one
     // quadrant at a time (the FP64 product's hi and lo tables)
-    const bool sl2l = ql2l || (!top && Pp * P <= TSIZE && P <= 64 && Pp <= PF_NCOEF);
+    const bool sl2l = ql2l || (!top && !dl2l && Pp * P <= TSIZE && P <= 64 && Pp <= PF_NCOEF);
     if (sl2l && !ql2l) l2l_staged(a, l, nl2l, wfirst, wstride, sT, wsm, lane, bid);
-    const int nm2l = (wpair && !tcl) ? a.npair[l] : 0;
+    const int nm2l = (wpair && !tcl) ? a.npair[l] * (ksh > 0 ? ksh * NH : 1) : 0;
     const int jst = nbst + l - 1;
     const int r0 = a.near_first ? (jst == 0 ? 0 : NI) : (int)((int64_t)NI * jst / nst);
     const int r1 = a.near_first ? NI : (int)((int64_t)NI * (jst + 1) / nst);
@@ -2428,6 +2670,19 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
             acc += A[(size_t)m * S] * ldcg(a.L[l - 1] + (size_t)par * Sp + Op + m);
           acc = wsum(acc);
           if (lane == 0) atomic_add(a.L[l] + (size_t)box * S + O + n, acc);
+        } else if (dl2l) {
+          const int box = a.ne[l][i / NH], par = box >> 2, q = box & 3, n = 32 * (i % NH) + lane;
+          const int S = a.S[l], O = a.O[l], Sp = a.S[l - 1], Op = a.O[l - 1];
+          float4* w = reinterpret_cast<float4*>(wsm);
+          __syncwarp();
+          for (int m = lane; m < Pp; m += 32) w[m] = dd_word(to_d(ldcg(a.L[l - 1] + (size_t)par * Sp + Op + m)));
+          __syncwarp();
+          if (n < P) {
+            const size_t o = (size_t)(q * Sp + Op) * S + O + n;
+            dflt re{0, 0}, im{0, 0};
+            dd_rows(re, im, a.l2lh[l - 1] + o, a.l2ll[l - 1] + o, S, w, Pp);
+            atomic_add(a.L[l] + (size_t)box * S + O + n, from_d<C>(cplx{dd_value(re), dd_value(im)}));
+          }
         } else {
           // the generic form, with the offsets of the used coefficients (see M2M)
           const int box = a.ne[l][i], par = box >> 2, q = box & 3;
@@ -2441,33 +2696,29 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
         }
         continue;
       }
-      const int pi = i - nl2l;
-      const int src = a.pr_src[l][pi], tgt = a.pr_tgt[l][pi];
-      const C phs = from_d<C>(phase_m(a.alpha, a.pr_img[l][pi]));
-      if (a.m2ltl[l]) {
-        // the FP64 product in double-float arithmetic on the FP32 pipes: the
-        // phased source multipole split into hi and lo parts, the operator
-        // read from its hi and lo tables
-        cplxf* wh = reinterpret_cast<cplxf*>(wsm);
-        cplxf* wl = wh + PF_NCOEF;
+      if (F64 && ksh > 0) {
+        // double-float arithmetic: the phased source multipole split into hi and lo
+        // parts, the operator rows m0 .. m1 read from its hi and lo tables
+        const int k = i - nl2l, sh = k % (ksh * NH), pi = k / (ksh * NH);
+        const int n = 32 * (sh % NH) + lane, q = sh / NH, m0 = P * q / ksh, m1 = P * (q + 1) / ksh;
+        const int src = a.pr_src[l][pi], tgt = a.pr_tgt[l][pi];
+        const int img = a.pr_img[l][pi];
+        const size_t o = ((size_t)a.pr_off[l][pi] * P + m0) * P + n;
+        float4* w = reinterpret_cast<float4*>(wsm);
         __syncwarp();
-        for (int m = lane; m < P; m += 32) {
-          const cplx v = to_d(phs * ldcg(a.M[l] + (size_t)src * P + m));
-          wh[m] = cplxf{(float)v.re, (float)v.im};
-          wl[m] = split_lo(v);
-        }
+        for (int m = m0 + lane; m < m1; m += 32)
+          w[m - m0] = dd_phase(a.alpha_w, img, __ldcg(a.Mw[l] + (size_t)src * P + m));
         __syncwarp();
-        const size_t ob = (size_t)a.pr_off[l][pi] * P * P;
-        const cplxf* Th = a.m2lth[l] + ob;
-        const cplxf* Tl = a.m2ltl[l] + ob;
-        for (int n = lane; n < P; n += 32) {
+        if (n < P) {
           dflt re{0, 0}, im{0, 0};
-#pragma unroll 4
-          for (int m = 0; m < P; ++m) dd_cmac(re, im, Th[(size_t)m * P + n], Tl[(size_t)m * P + n], wh[m], wl[m]);
+          dd_rows(re, im, a.m2lth[l] + o, a.m2ltl[l] + o, P, w, m1 - m0);
           atomic_add(a.L[l] + (size_t)tgt * P + n, from_d<C>(cplx{dd_value(re), dd_value(im)}));
         }
         continue;
       }
+      const int pi = i - nl2l;
+      const int src = a.pr_src[l][pi], tgt = a.pr_tgt[l][pi];
+      const C phs = from_d<C>(phase_m(a.alpha, a.pr_img[l][pi]));
       const int S = a.S[l], O = a.O[l];
       const C* To = a.m2lt[l] + (size_t)a.pr_off[l][pi] * S * S + (size_t)O * S + O;
       __syncwarp();
@@ -2491,7 +2742,58 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
   {
     const int PD = a.P[D], SD = a.S[D], OD = a.O[D];
     const C c2 = from_d<C>(a.c2);
-    const int nit = (a.E + 31) >> 5;
+    // FP64 product in double-float arithmetic: a warp takes 16 elements of one leaf,
+    // the lanes over the elements and the two halves of the coefficients; the leaf's
+    // expansion is split into its parts once per warp
+    if (F64 && a.l2pl && PD <= PF_NCOEF) {
+      float4* w = reinterpret_cast<float4*>(wsm);
+      const int el = lane & 15, hf = lane >> 4, t0 = hf ? (PD + 1) / 2 : 0, t1 = hf ? PD : (PD + 1) / 2;
+      constexpr int NS = 4;                       // items per leaf (more elements: further passes)
+      for (int i = wfirst; i < NS * a.nne[D]; i += wstride) {
+        const int box = a.ne[D][i / NS], s0 = a.bb[D][box], s1 = a.be[D][box];
+        if (s0 + 16 * (i % NS) >= s1) continue;
+        __syncwarp();
+        for (int m = lane; m < PD; m += 32) w[m] = dd_word(to_d(ldcg(a.L[D] + (size_t)box * PD + m)));
+        __syncwarp();
+        for (int sb = s0 + 16 * (i % NS); sb < s1; sb += 16 * NS) {
+          const int s = sb + el;
+          const bool on = s < s1;
+          const size_t o = on ? s : s1 - 1;
+          const cplxf *ch = a.l2ph + o, *cl = a.l2pl + o;
+          dflt ur{0, 0}, ui{0, 0}, dr{0, 0}, di{0, 0};
+#pragma unroll 5
+          for (int t = t0; t < t1; ++t) {
+            const float4 v = w[t];
+            const cplxf Lh{v.x, v.y}, Ll{v.z, v.w};
+            const size_t k0 = (size_t)t * a.E, k1 = (size_t)(PD + t) * a.E;
+            dd_cmac(ur, ui, ch[k0], cl[k0], Lh, Ll);
+            dd_cmac(dr, di, ch[k1], cl[k1], Lh, Ll);
+          }
+          auto both = [](dflt v) {
+            return dd_add(v, dflt{__shfl_down_sync(0xffffffffu, v.h, 16), __shfl_down_sync(0xffffffffu, v.l, 16)});
+          };
+          ur = both(ur);
+          ui = both(ui);
+          dr = both(dr);
+          di = both(di);
+          if (hf == 0 && on) {
+            const int e = a.perm[s];
+            const cplx po = conj(a.ph[s]);
+            const float4* Un = reinterpret_cast<const float4*>(a.Un) + 2 * (size_t)s;
+            const float4 n0 = __ldcg(Un), n1 = __ldcg(Un + 1);
+            ur = dd_add(ur, dflt{n0.x, n0.z});
+            ui = dd_add(ui, dflt{n0.y, n0.w});
+            dr = dd_add(dr, dflt{n1.x, n1.z});
+            di = dd_add(di, dflt{n1.y, n1.w});
+            const cplx u = po * cplx{dd_value(ur), dd_value(ui)};
+            const cplx du = a.c2 * (po * cplx{dd_value(dr), dd_value(di)});
+            a.y[2 * e] = ldcg(a.y + 2 * e) + u;
+            a.y[2 * e + 1] = ldcg(a.y + 2 * e + 1) + du;
+          }
+        }
+      }
+    }
+    const int nit = F64 && a.l2pl && PD <= PF_NCOEF ? 0 : (a.E + 31) >> 5;
     for (int it = wfirst; it < nit; it += wstride) {
       const int s = (it << 5) + lane;
       if (s >= a.E) continue;
@@ -2499,21 +2801,7 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
       const C* Lb = a.L[D] + (size_t)box * SD + OD;
       const C* cs = a.l2p + s + (size_t)OD * a.E;
       C uf{0, 0}, df{0, 0};
-      if (a.l2pl && a.l2p_dd) {
-        // FP64 product: L2P in double-float arithmetic from the caches' hi and lo parts
-        const cplxf* ch = a.l2ph + s + (size_t)OD * a.E;
-        const cplxf* cl = a.l2pl + s + (size_t)OD * a.E;
-        dflt ur{0, 0}, ui{0, 0}, dr{0, 0}, di{0, 0};
-#pragma unroll 8
-        for (int t = 0; t < PD; ++t) {
-          const cplx Lt = to_d(ldcg(Lb + t));
-          const cplxf Lh{(float)Lt.re, (float)Lt.im}, Ll = split_lo(Lt);
-          dd_cmac(ur, ui, ch[(size_t)t * a.E], cl[(size_t)t * a.E], Lh, Ll);
-          dd_cmac(dr, di, ch[(size_t)(SD + t) * a.E], cl[(size_t)(SD + t) * a.E], Lh, Ll);
-        }
-        uf = from_d<C>(cplx{dd_value(ur), dd_value(ui)});
-        df = from_d<C>(cplx{dd_value(dr), dd_value(di)});
-      } else {
+      {
 #pragma unroll 16
         for (int t = 0; t < PD; ++t) {
           const C Lt = ldcg(Lb + t);
@@ -2686,11 +2974,14 @@ cudaError_t fill_args(pfmbem* h, const cplx* x, cplx* y, const int* done, FusedA
       cudaError_t e = k_near64(h);                  // FP64 blocks, formed on first use
       if (e != cudaSuccess) return e;
     }
-    if (h->nc_vall && h->dens_dd && !near64) {
+    if (h->nc_vall && h->dens_dd && h->l2p_cl && h->p2m_cl && !near64) {
       a.nc_lo = h->nc_vall;
       a.nc_hi = h->nc_valf;
       a.dens_dd = h->dens_dd;
+      const cplxf ah = to_f(h->alpha), alo = split_lo(h->alpha);
+      a.alpha_w = make_float4(ah.re, ah.im, alo.re, alo.im);
       for (int l = 1; l <= h->D; ++l) {
+        a.Mw[l] = h->lev[l].Mw;
         a.m2lth[l] = h->lev[l].m2ltf;
         a.m2ltl[l] = h->lev[l].m2ltl;
       }
@@ -2704,12 +2995,8 @@ cudaError_t fill_args(pfmbem* h, const cplx* x, cplx* y, const int* done, FusedA
       }
       a.p2mh = h->p2m_cf;
       a.p2ml = h->p2m_cl;
-      if (h->l2p_cl) {
-        a.l2ph = h->l2p_cf;
-        a.l2pl = h->l2p_cl;
-        static const bool l2pdd = std::getenv("PFMBEM_L2P_DD") != nullptr;
-        a.l2p_dd = l2pdd ? 1 : 0;
-      }
+      a.l2ph = h->l2p_cf;
+      a.l2pl = h->l2p_cl;
     }
     a.m2m31 = h->m2m31; a.root1 = h->root1;
     a.nc_val = h->nc_val; a.fb_val = h->fb_val; a.fh_val = h->fh_val; a.tw = h->tw;
@@ -2758,14 +3045,16 @@ cudaError_t launch_fused(pfmbem* h, const cplx* x, cplx* y, bool f32, const int*
   // against the P2M warp items (one leaf per warp)
   {
     const int nf = h->fz_nfft + h->fz_nchunk;
-    const double wa = (double)h->lev[h->D].nne / nwarp;
+    // (the FP64 product's P2M, two double-float warps a leaf, weighs 2.65 times as much:
+    // on the 32x32 block 304 fiber blocks were done in 63 us, the other 152 in 180)
+    const double wa = (f32 ? 1.0 : 2.65) * (double)h->lev[h->D].nne / nwarp;
     const int fb = (int)((double)grid * nf / (nf + wa) + 0.5);
     a.fblk = grid >= 16 ? std::max(1, std::min({fb, nf, grid - grid / 4})) : 0;
   }
-  // M2L: warp per pair in FP64, whose per-pair cost the FP64 pipe sets; staged
-  // chunks in FP32 (PFMBEM_M2L_WARP=0/1 overrides, for measurement)
+  // M2L in staged chunks, or one warp per pair where the FP64 product has no
+  // double-float tables (PFMBEM_M2L_WARP=0/1 overrides, for measurement)
   static const char* mw = std::getenv("PFMBEM_M2L_WARP");
-  a.m2l_warp = mw ? std::atoi(mw) != 0 : !f32;
+  a.m2l_warp = mw ? std::atoi(mw) != 0 : !f32 && !a.nc_lo;
   static const bool nf = std::getenv("PFMBEM_NEAR_FIRST") != nullptr;
   a.near_first = nf ? 1 : 0;
   // levels 1 and 0 inside the level-2 stage when the tree has level 3 and the
@@ -3148,6 +3437,10 @@ cudaError_t k_fused_prepare(pfmbem* h, bool* ok) {
   // leaves and over fibers or fiber row chunks (fiber part of A)
   int need = std::max(h->lev[h->D].nne, h->fz_nchunk + h->fz_nfft);
   for (int l = 0; l <= h->D; ++l) need = std::max(need, (h->lev[l].nne + FW - 1) / FW);
+  // and the near-field rows (a warp each) and M2L chunks (a block each): a small
+  // block's product is a chain of latencies, shorter over more SMs
+  need = std::max(need, (h->E + FW - 1) / FW);
+  for (int l = 1; l <= h->D; ++l) need = std::max(need, h->lev[l].nchunk);
   need = std::max(need, 1);
   // staging region of the FP32 product: room for the four stacked quadrant
   // operators of M2M and L2L at the FP32 orders, within about 100 KB per block
