@@ -115,6 +115,7 @@ struct FusedArgs {
   const int4* nr_piece;
   int npiece;
   const int* nc_src;
+  int64_t near_blocks;               // near-field 2 x 2 blocks in all
   const C* nc_val;
   int nchunk;                        // direct-row chunks (fibers not applied by FFT)
   const int* fb_chunk;
@@ -708,6 +709,10 @@ __device__ __noinline__ void near_row_dd(const FusedArgs<C>& a, int s, int lane)
     const float4 h = __ldcg(dh + f), l = __ldcg(dl + f);
     const float4 h0 = __ldg(qh + 2 * j), h1 = __ldg(qh + 2 * j + 1), l0 = __ldg(ql + 2 * j), l1 = __ldg(ql + 2 * j + 1);
     f = j + 32 < ns ? __ldg(src + j + 32) : 0;
+    if ((lane & 3) == 0 && j + 64 < ns) {           // the pass after next, into L2
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(qh + 2 * (j + 64)));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(ql + 2 * (j + 64)));
+    }
     const cplxf ph{h.x, h.y}, pl{l.x, l.y}, vh{h.z, h.w}, vl{l.z, l.w};
     dd_cmac(ur, ui, cplxf{h0.x, h0.y}, cplxf{l0.x, l0.y}, ph, pl);
     dd_cmac(dr, di, cplxf{h1.x, h1.y}, cplxf{l1.x, l1.y}, ph, pl);
@@ -830,58 +835,84 @@ __device__ __forceinline__ void near_row(const FusedArgs<C>& a, int s, int lane)
 // The descriptor d (read ahead by the stage loops) holds everything the piece
 // needs to start: its block offset, its first source and (count, target).
 constexpr int NR_PIECE = 128;
+// All loads are 16 bytes (a block's four entries are 32, a source's two hi or lo parts
+// 16), and the four sums share their reduction (near_sum4).
+__device__ __forceinline__ int64_t piece_row(int4 d) {
+  return (int64_t)(((unsigned long long)(unsigned)d.y << 32) | (unsigned)d.x);
+}
+// Sums over the warp of four values; lanes 0, 8, 16, 24 return those of a, b, c, d.
+__device__ __forceinline__ float near_sum4(float a, float b, float c, float d, int lane) {
+  const bool u = (lane & 16) != 0, v = (lane & 8) != 0;
+  const float p = (u ? c : a) + __shfl_xor_sync(0xffffffffu, u ? a : c, 16);
+  const float q = (u ? d : b) + __shfl_xor_sync(0xffffffffu, u ? b : d, 16);
+  float r = (v ? q : p) + __shfl_xor_sync(0xffffffffu, v ? p : q, 8);
+  r += __shfl_xor_sync(0xffffffffu, r, 4);
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  return r + __shfl_xor_sync(0xffffffffu, r, 1);
+}
 __device__ __forceinline__ void near_piece_diff(const FusedArgs<cplxf>& a, int4 d, int lane) {
-  const int64_t r = (int64_t)(((unsigned long long)(unsigned)d.y << 32) | (unsigned)d.x);
   const int cnt = (int)((unsigned)d.w >> 24), s = (int)((unsigned)d.w & 0xffffffu);
-  const cplxf* row = a.nc_val + r;
+  const float4* row = reinterpret_cast<const float4*>(a.nc_val + piece_row(d));
+  const float4* dh = reinterpret_cast<const float4*>(a.dens);
+  const float4* dl = reinterpret_cast<const float4*>(a.dlo);
   const int* src = a.nc_src + d.z;
-  const cplxf tph = ldcg(a.dens + 2 * s), tpl = ldcg(a.dlo + 2 * s);
-  const cplxf tvh = ldcg(a.dens + 2 * s + 1), tvl = ldcg(a.dlo + 2 * s + 1);
+  const float4 th = __ldcg(dh + s), tl = __ldcg(dl + s);
   constexpr int NJ = NR_PIECE / 32;
   int f[NJ];
-  cplxf q[NJ][4];
+  float4 q0[NJ], q1[NJ];
 #pragma unroll
   for (int k = 0; k < NJ; ++k) {
     const int jj = lane + 32 * k;
-    f[k] = jj < cnt ? __ldg(src + jj) : s;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) q[k][c] = jj < cnt ? row[4 * jj + c] : cplxf{0, 0};
+    const bool on = jj < cnt;
+    f[k] = on ? __ldg(src + jj) : s;
+    q0[k] = on ? __ldg(row + 2 * jj) : make_float4(0.f, 0.f, 0.f, 0.f);
+    q1[k] = on ? __ldg(row + 2 * jj + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   cplxf u0{0, 0}, d0{0, 0}, u1{0, 0}, d1{0, 0};
 #pragma unroll
-  for (int k = 0; k < NJ; k += 2) {
-    const cplxf p0 = (ldcg(a.dens + 2 * f[k]) - tph) + (ldcg(a.dlo + 2 * f[k]) - tpl);
-    const cplxf v0 = (ldcg(a.dens + 2 * f[k] + 1) - tvh) + (ldcg(a.dlo + 2 * f[k] + 1) - tvl);
-    const cplxf p1 = (ldcg(a.dens + 2 * f[k + 1]) - tph) + (ldcg(a.dlo + 2 * f[k + 1]) - tpl);
-    const cplxf v1 = (ldcg(a.dens + 2 * f[k + 1] + 1) - tvh) + (ldcg(a.dlo + 2 * f[k + 1] + 1) - tvl);
-    u0 += q[k][0] * p0 + q[k][1] * v0;
-    d0 += q[k][2] * p0 + q[k][3] * v0;
-    u1 += q[k + 1][0] * p1 + q[k + 1][1] * v1;
-    d1 += q[k + 1][2] * p1 + q[k + 1][3] * v1;
+  for (int k = 0; k < NJ; ++k) {
+    const float4 h = __ldcg(dh + f[k]), l = __ldcg(dl + f[k]);
+    const cplxf p{(h.x - th.x) + (l.x - tl.x), (h.y - th.y) + (l.y - tl.y)};
+    const cplxf v{(h.z - th.z) + (l.z - tl.z), (h.w - th.w) + (l.w - tl.w)};
+    const cplxf u = cplxf{q0[k].x, q0[k].y} * p + cplxf{q0[k].z, q0[k].w} * v;
+    const cplxf w = cplxf{q1[k].x, q1[k].y} * p + cplxf{q1[k].z, q1[k].w} * v;
+    if (k & 1) {
+      u1 += u;
+      d1 += w;
+    } else {
+      u0 += u;
+      d0 += w;
+    }
   }
-  const cplxf u = wsum(u0 + u1), du = wsum(d0 + d1);
-  if (lane == 0 && cnt > 0) {
-    atomic_add(a.Un + 2 * s, u);
-    atomic_add(a.Un + 2 * s + 1, du);
-  }
+  u0 += u1;
+  d0 += d1;
+  const float r = near_sum4(u0.re, u0.im, d0.re, d0.im, lane);
+  const float r1 = __shfl_down_sync(0xffffffffu, r, 8);       // the imaginary part, on lanes 0 and 16
+  if ((lane & 15) == 0 && cnt > 0) atomic_add(a.Un + 2 * s + (lane >> 4), cplxf{r, r1});
 }
 
 // The near items [ifirst, nitem) of a stage that fall to one warp (every
 // wstride-th from its first), item i being near item r0 + i - base: pieces
-// (FP32 product in differences) with the next descriptor read while the current
-// piece runs, so that a piece costs about two dependent loads instead of four;
-// else whole rows.  nd: the warp's first descriptor, read by the caller before
-// the stage's box items.
+// (FP32 product in differences) with the descriptors of the next two read while the
+// current piece runs, so that a piece costs about two dependent loads instead of four,
+// and the next piece's blocks asked into the L2 (where they do not fit it, a piece
+// otherwise waits for DRAM); else whole rows.  nd: the warp's first descriptor, read
+// by the caller before the stage's box items.
 template <class C>
 __device__ __forceinline__ void near_items(const FusedArgs<C>& a, int ifirst, int nitem, int wstride, int r0,
                                            int base, int4 nd, int lane) {
   if constexpr (sizeof(C) == sizeof(cplxf)) {
     if (a.npiece > 0) {
+      const int4* pc = a.nr_piece + (r0 - base);
+      int4 n1 = ifirst + wstride < nitem ? __ldg(pc + ifirst + wstride) : int4{0, 0, 0, 0};
       for (int i = ifirst; i < nitem; i += wstride) {
-        const int in = i + wstride;
-        const int4 dn = in < nitem ? __ldg(a.nr_piece + r0 + (in - base)) : nd;
+        const int in = i + 2 * wstride;
+        const int4 n2 = in < nitem ? __ldg(pc + in) : int4{0, 0, 0, 0};
+        if (4 * lane < (int)((unsigned)n1.w >> 24))
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(a.nc_val + piece_row(n1) + 16 * lane));
         near_piece_diff(a, nd, lane);
-        nd = dn;
+        nd = n1;
+        n1 = n2;
       }
       return;
     }
@@ -1812,10 +1843,12 @@ __device__ bool tc_m2l_item(const FusedArgs<cplxf>& a, int l, int item, unsigned
   return true;
 }
 
-// Asks the L2 for `bytes` from p on, a line per thread of the G blocks: the tables of
-// the next stage, which the near-field stream (more than the L2 holds in the FP64
-// product) has pushed out since the last product; every load of a stage that misses
-// would wait for DRAM in a chain of a few such batches.
+// Asks the L2 for `bytes` from p on, a line per thread of the G blocks: the FP64
+// product's tables of the next stage, which its near-field stream (with the tables more
+// than the L2 holds: 190 MB on the 8x8 hexagon block) has pushed out since the last
+// product; every load of a stage that misses would wait for DRAM in a chain of a few
+// such batches (389 -> 316 us there, with the near blocks below).  The FP32 product's
+// working set of such a block stays in the L2 and gains nothing (156 -> 167 us).
 __device__ __forceinline__ void l2_prefetch(const void* p, size_t bytes, int bid, int G) {
   const char* c = static_cast<const char*>(p);
   for (size_t o = ((size_t)bid * nt() + threadIdx.x) * 128; o < bytes; o += (size_t)G * nt() * 128)
@@ -1828,8 +1861,6 @@ __device__ __forceinline__ void prefetch_m2m(const FusedArgs<C>& a, int l, int b
   if (sizeof(C) == sizeof(cplx) && a.m2ml[l]) {
     l2_prefetch(a.m2mh[l], n, bid, G);
     l2_prefetch(a.m2ml[l], n, bid, G);
-  } else {
-    l2_prefetch(a.m2m[l], n / sizeof(cplxf) * sizeof(C), bid, G);
   }
 }
 template <class C>
@@ -1842,9 +1873,6 @@ __device__ __forceinline__ void prefetch_down(const FusedArgs<C>& a, int l, int 
       l2_prefetch(a.l2lh[l - 1], nl, bid, G);
       l2_prefetch(a.l2ll[l - 1], nl, bid, G);
     }
-  } else if (sizeof(C) == sizeof(cplxf)) {
-    l2_prefetch(a.m2lt[l], n, bid, G);
-    l2_prefetch(a.l2l[l - 1], nl, bid, G);
   }
 }
 template <class C>
@@ -1853,11 +1881,36 @@ __device__ __forceinline__ void prefetch_l2p(const FusedArgs<C>& a, int bid, int
   if (sizeof(C) == sizeof(cplx) && a.l2pl) {
     l2_prefetch(a.l2ph, n, bid, G);
     l2_prefetch(a.l2pl, n, bid, G);
-  } else if (sizeof(C) == sizeof(cplxf)) {
-    const int O = a.O[a.D];
-    l2_prefetch(a.l2p + (size_t)O * a.E, n / 2, bid, G);
-    l2_prefetch(a.l2p + (size_t)(a.S[a.D] + O) * a.E, n / 2, bid, G);
   }
+}
+
+// The near-field blocks of the warp items of stage j of nst, about their share of the
+// array (rows are dealt by number, not by bytes), where that is no more than 16 MB.
+template <class C>
+__device__ __forceinline__ void prefetch_near(const FusedArgs<C>& a, int j, int nst, int bid, int G) {
+  const size_t n = (size_t)a.near_blocks * 4 * sizeof(cplxf), o0 = n / nst * j & ~(size_t)127;
+  const size_t len = min(n / nst, n - o0);
+  if (len > (size_t)16 << 20) return;
+  if (sizeof(C) == sizeof(cplx) && a.nc_lo) {
+    l2_prefetch(reinterpret_cast<const char*>(a.nc_hi) + o0, len, bid, G);
+    l2_prefetch(reinterpret_cast<const char*>(a.nc_lo) + o0, len, bid, G);
+  }
+}
+
+// Who takes a stage's W warp items when its N block items do not come out even over
+// the G blocks: the blocks with one block item less, if that ends sooner than all of
+// them (in units of a warp item, a block item takes R).  A block that carries an
+// operator's copy and its boxes then goes straight to the barrier instead of on to
+// near-field rows, which used to make it the stage's last.
+template <class C>
+__device__ __forceinline__ void warp_share(int N, int W, int rank, int warp, int G, int& wf, int& ws) {
+  constexpr int R = sizeof(C) == sizeof(cplx) ? 3 : 1;
+  const int q = N / G, e = N - q * G;
+  if (e == 0) return;
+  const int ra = (W + G * nw() - 1) / (G * nw()), rr = (W + (G - e) * nw() - 1) / ((G - e) * nw());
+  if (max((q + 1) * R, q * R + rr) >= (q + 1) * R + ra) return;
+  ws = (G - e) * nw();
+  wf = rank < e ? W : warp_first(rank - e, warp, G - e);
 }
 
 // Block items of the next stage, so that a block can stage their operators in
@@ -2228,6 +2281,7 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
       prefetch_m2m(a, D - 1, bid, G);
     else
       prefetch_down(a, 1, bid, G);
+    prefetch_near(a, 0, D - (a.top3 ? 2 : 0) + D, bid, G);
     for (int l = 1; l <= D; ++l) {
       C* Lz = a.L[l];
       const size_t nz = (size_t)a.nbox[l] * a.S[l];
@@ -2393,6 +2447,7 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
   for (int l = D - 1; l >= lstop; --l) {
     const int P = a.P[l], Pc = a.P[l + 1];
     const int jst = D - 1 - l;
+    prefetch_near(a, jst + 1, nst, bid, G);
     if (l - 1 >= lstop)
       prefetch_m2m(a, l - 1, bid, G);
     else
@@ -2425,9 +2480,14 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
     else if (staged)
       m2m_staged(a, l, nbi, wfirst, wstride, sT, wsm, lane, bid);
     if (a.bdone && threadIdx.x == 0) a.bdone[(size_t)(ks - 1) * G + bid] = gtimer();
+    int wf = wfirst, ws = wstride;
+    if (split || quad)
+      warp_share<C>(split ? nbi : (nbi + nw() - 1) / nw(), nx + (r1 - r0), rank(ks - 1), warp, G, wf, ws);
+    // (with the boxes as block items, the warp items start at nbi)
+    const int w0 = split || quad ? nbi : 0;
     int4 nd;
-    const int inear = first_near(a, wfirst, wstride, nbi + nx, nitem, r0, &nd);
-    for (int i = wfirst; i < nbi + nx; i += wstride) {
+    const int inear = first_near(a, w0 + wf, ws, nbi + nx, nitem, r0, &nd);
+    for (int i = w0 + wf; i < nbi + nx; i += ws) {
       if (staged && i < nbi) continue;
       if (i >= nbi) {
         // M(1) of a level-1 box from its 16 level-3 boxes; the multipoles of
@@ -2537,7 +2597,7 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
         }
       }
     }
-    near_items(a, inear, nitem, wstride, r0, nbi + nx, nd, lane);
+    near_items(a, inear, nitem, ws, r0, nbi + nx, nd, lane);
     // the next stage's operators, staged ahead (this stage's items are done
     // with the shared memory once the block has passed this point)
     if (l - 1 >= lstop)
@@ -2554,10 +2614,12 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
   // ------------------------------------------------------------ D: L2L + M2L
   for (int l = 1; l <= D; ++l) {
     const int P = a.P[l], Pp = a.P[l - 1];
-    if (l < D)
+    if (l < D) {
+      prefetch_near(a, nbst + l, nst, bid, G);
       prefetch_down(a, l + 1, bid, G);
-    else
+    } else {
       prefetch_l2p(a, bid, G);
+    }
     // L2L: one warp per output coefficient while the boxes are few, else one
     // warp per box
     const bool top = (int64_t)a.nne[l] * P <= wstride;
@@ -2642,9 +2704,12 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
     const int r0 = a.near_first ? (jst == 0 ? 0 : NI) : (int)((int64_t)NI * jst / nst);
     const int r1 = a.near_first ? NI : (int)((int64_t)NI * (jst + 1) / nst);
     const int nitem = nl2l + nm2l + (r1 - r0);
+    int wf = wfirst, ws = wstride;
+    const int w0 = sl2l ? nl2l : 0;                    // L2L as block items: the warp items start after it
+    warp_share<C>(ntc + nchu + ngl, nitem - w0, rank(ks - 1), warp, G, wf, ws);
     int4 nd;
-    const int inear = first_near(a, wfirst, wstride, nl2l + nm2l, nitem, r0, &nd);
-    for (int i = wfirst; i < nl2l + nm2l; i += wstride) {
+    const int inear = first_near(a, w0 + wf, ws, nl2l + nm2l, nitem, r0, &nd);
+    for (int i = w0 + wf; i < nl2l + nm2l; i += ws) {
       if (i < nl2l) {
         if (sl2l) continue;
         if (top && a.top3 && l == 1) {
@@ -2726,7 +2791,7 @@ __device__ __forceinline__ bool fused_body(const FusedArgs<C>& a, const int bid,
       __syncwarp();
       for (int n = lane; n < P; n += 32) atomic_add(a.L[l] + (size_t)tgt * S + O + n, colmv(To + n, S, wsm, P));
     }
-    near_items(a, inear, nitem, wstride, r0, nl2l + nm2l, nd, lane);
+    near_items(a, inear, nitem, ws, r0, nl2l + nm2l, nd, lane);
     if (l < D) prefetch(ks, -1, l + 1);     // the next D stage's operators, staged ahead
     if (!group_barrier(a.bar, a.err, a.wait_ns, G, bid, a.arrive ? a.arrive + (size_t)(ks - 1) * G : nullptr)) {
       tc_leave();
@@ -3004,6 +3069,7 @@ cudaError_t fill_args(pfmbem* h, const cplx* x, cplx* y, const int* done, FusedA
   a.nc_base = h->nc_base;
   a.nc_sbase = h->nc_sbase;
   a.nc_src = h->nc_src;
+  a.near_blocks = h->nc_blocks;
   a.nchunk = h->fz_nchunk;
   a.fb_chunk = h->fz_chunk;
   a.nfft = h->fz_nfft;
