@@ -591,23 +591,24 @@ __global__ void root1_kernel(int P0, int P1, const cplx* __restrict__ l2l0, cons
 
 // ------------------------------------------------------------ double-float sums
 // A value h + l held as two FP32 numbers (about 48 bits).  acc += a b with
-// a = ah + al, b = bh + bl: the product ah bh exactly as p + e (one rounding,
-// its error by a fused multiply-add), the cross terms ah bl + al bh into e, and
-// p added to acc.h by the two-sum of Knuth, whose error goes to acc.l with e.
-// Explicitly rounded intrinsics keep the compiler from contracting the steps.
+// a = ah + al, b = bh + bl: p = ah bh rounded enters acc.h by the two-sum of Knuth
+// (s = h + p, v = s - h; the errors h - (s - v) and p - v are exact), and one fused
+// multiply-add ah bh - v gives p - v together with the rounding error of p, so the
+// sum's second error and the product's error cost one instruction; the cross terms
+// ah bl + al bh join it.  Ten FP32 instructions, which bound the translations (twelve
+// with the two errors formed apart).  Explicitly rounded intrinsics keep the compiler
+// from contracting the steps.
 struct dflt {
   float h, l;
 };
 
 __device__ __forceinline__ void dd_mac(dflt& acc, float ah, float al, float bh, float bl) {
-  const float p = __fmul_rn(ah, bh);
-  float e = __fmaf_rn(ah, bh, -p);
-  e = __fmaf_rn(ah, bl, __fmaf_rn(al, bh, e));
-  const float s = __fadd_rn(acc.h, p);
+  const float s = __fadd_rn(acc.h, __fmul_rn(ah, bh));
   const float v = __fsub_rn(s, acc.h);
-  const float err = __fadd_rn(__fsub_rn(acc.h, __fsub_rn(s, v)), __fsub_rn(p, v));
+  const float d = __fsub_rn(acc.h, __fsub_rn(s, v));
+  const float e = __fmaf_rn(ah, bl, __fmaf_rn(al, bh, __fmaf_rn(ah, bh, -v)));
   acc.h = s;
-  acc.l = __fadd_rn(acc.l, __fadd_rn(err, e));
+  acc.l = __fadd_rn(acc.l, __fadd_rn(d, e));
 }
 
 // acc += a b for complex a, b given as hi and lo parts
