@@ -451,7 +451,13 @@ cudaError_t k_tri_caches(pfmbem* h);
 // Triangle tree: level l's M2L operator as hi and lo parts, and its M2L by
 // offset groups in double-float arithmetic (matvec_fused.cu).
 cudaError_t k_tri_m2l_split(pfmbem* h, int l);
-cudaError_t k_tri_m2l_dd(pfmbem* h, int l);
+cudaError_t k_tri_m2l_dd(pfmbem* h);
+size_t k_tri_m2l_smem(int P);
+constexpr size_t TRI_M2L_SMEM = 200 * 1024;   // above it a level's M2L goes target by target
+cudaError_t k_tri_words(pfmbem* h);
+cudaError_t k_tri_top(pfmbem* h, cudaStream_t st);
+cudaError_t k_tri_fiber(pfmbem* h, const cplx* x, cplx* y, cudaStream_t st);
+cudaError_t k_tri_l2p(pfmbem* h, cplx* y);
 // Triangle tree: M2M of level l from level l + 1, and L2L of level l from l - 1,
 // in double-float arithmetic.
 cudaError_t k_tri_m2m_dd(pfmbem* h, int l);

@@ -1861,13 +1861,15 @@ __global__ void gather_t_kernel(int E, const int* __restrict__ perm, const cplx*
 }
 
 // M(leaf)_n = sum_f c[f][0][n] phi'_f + c[f][1][n] varphi'_f; one block per leaf.
+// Clears L(leaf) where Lz is given (the triangle tree's M2L adds to it).
 template <class C>
 __global__ void p2m_apply_t_kernel(const int* __restrict__ ne, const int* __restrict__ bb,
                                    const int* __restrict__ be, int P, const C* __restrict__ coef,
-                                   const C* __restrict__ dens, C* __restrict__ Mout) {
+                                   const C* __restrict__ dens, C* __restrict__ Mout, C* __restrict__ Lz = nullptr) {
   const int box = ne[blockIdx.x];
   const int n = threadIdx.x;
   if (n >= P) return;
+  if (Lz) Lz[(size_t)box * P + n] = C{0, 0};
   C acc{0, 0};
   for (int f = bb[box]; f < be[box]; ++f) {
     const C* cf = coef + (size_t)f * 2 * P;
@@ -2407,6 +2409,14 @@ cudaError_t k_near64(pfmbem* h) {
 // are tree-independent (P2M/L2P coefficients at the leaves' centroids, near-field
 // and same-fiber blocks, M2L by offset groups), and M2M/L2L with the per-box
 // operators of the triangles.
+// Two chains that meet at the end.  The tree's translations keep the FP32 pipes
+// busy (double-float M2M, M2L, L2L); the near-field and same-fiber blocks and the
+// operator between the cells are FP64 sums and table reads, and run beside them on
+// the handle's second stream: near sums and same-fiber rows (which write y) while the
+// tree works upward and across, the cells' operator after the M2M; the L2L and L2P
+// (which adds to y) wait for that stream.  So M2L comes before L2L and adds
+// to expansions that the upward pass cleared.  16384 elements, p = 30: 1.78 ms as
+// one chain.
 static cudaError_t matvec_tri_cached(pfmbem* h, const cplx* x, cplx* y) {
   cudaStream_t st = h->stream;
   const int E = h->E, D = h->D;
@@ -2414,12 +2424,27 @@ static cudaError_t matvec_tri_cached(pfmbem* h, const cplx* x, cplx* y) {
   const cplx alpha = h->alpha;
   cudaError_t e = k_near64(h);
   if (e != cudaSuccess) return e;
+  // one chain where phases are timed, for their events lie on one stream
+  const bool fork = h->aux[0] && h->aux_ev[0] && h->fork_ev && h->side_ev && !h->prof.on;
+  cudaStream_t st2 = fork ? h->aux[0] : st;
   prof_begin(h, PH_GATHER);
   gather_dens_kernel<<<(E + 255) / 256, 256, 0, st>>>(E, h->s_perm, h->s_ph, x, h->dens);
   prof_end(h, PH_GATHER);
+  if (fork) {
+    if ((e = cudaEventRecord(h->fork_ev, st)) != cudaSuccess) return e;
+    if ((e = cudaStreamWaitEvent(st2, h->fork_ev, 0)) != cudaSuccess) return e;
+  }
+  prof_begin(h, PH_NEAR);
+  if ((e = cudaMemsetAsync(h->U, 0, 2 * sizeof(cplx) * (size_t)E, st2)) != cudaSuccess) return e;
+  near_apply_t_kernel<cplx><<<leaf.nne, 256, 0, st2>>>(leaf.ne, leaf.box_begin, leaf.box_end, h->nc_base, h->nc_sbase,
+                                                       h->nc_src, h->nc_val, h->dens, h->U);
+  prof_end(h, PH_NEAR);
+  prof_begin(h, PH_FIBER);
+  if ((e = k_tri_fiber(h, x, y, st2)) != cudaSuccess) return e;
+  prof_end(h, PH_FIBER);
   prof_begin(h, PH_P2M);
   p2m_apply_t_kernel<cplx><<<leaf.nne, round32(leaf.P), 0, st>>>(leaf.ne, leaf.box_begin, leaf.box_end, leaf.P,
-                                                                 h->p2m_c, h->dens, leaf.M);
+                                                                 h->p2m_c, h->dens, leaf.M, leaf.L);
   prof_end(h, PH_P2M);
   // M2M, L2L and M2L in double-float arithmetic on the FP32 pipes
   // (PFMBEM_TRI_M2L64=1: FP64 instructions, for measurement)
@@ -2428,7 +2453,7 @@ static cudaError_t matvec_tri_cached(pfmbem* h, const cplx* x, cplx* y) {
     Level& a = h->lev[l];
     Level& c = h->lev[l + 1];
     prof_begin(h, PH_M2M);
-    if (a.tri_m2m_hl && !m2l64) {
+    if (!m2l64) {
       e = k_tri_m2m_dd(h, l);
       if (e != cudaSuccess) return e;
     } else {
@@ -2437,22 +2462,31 @@ static cudaError_t matvec_tri_cached(pfmbem* h, const cplx* x, cplx* y) {
     }
     prof_end(h, PH_M2M);
   }
-  const int rows = h->nroot * h->lev[0].P;
+  if (fork) {
+    if ((e = cudaEventRecord(h->side_ev, st)) != cudaSuccess) return e;
+    if ((e = cudaStreamWaitEvent(st2, h->side_ev, 0)) != cudaSuccess) return e;
+  }
   prof_begin(h, PH_LOCAL);
-  top_apply_kernel<<<(rows * 32 + 255) / 256, 256, 0, st>>>(rows, h->root, h->lev[0].M, h->lev[0].L);
+  if ((e = k_tri_top(h, st2)) != cudaSuccess) return e;
   prof_end(h, PH_LOCAL);
+  if (fork && (e = cudaEventRecord(h->aux_ev[0], st2)) != cudaSuccess) return e;
   // M2L by offset groups; where a group's operator does not fit shared memory,
   // per target over its list, with L2L
+  auto grouped = [&](int l) { return !m2l64 && k_tri_m2l_smem(h->lev[l].P) <= TRI_M2L_SMEM; };
+  if (!m2l64) {
+    prof_begin(h, PH_M2L);
+    if ((e = k_tri_m2l_dd(h)) != cudaSuccess) return e;
+    prof_end(h, PH_M2L);
+  }
+  if (fork && (e = cudaStreamWaitEvent(st, h->aux_ev[0], 0)) != cudaSuccess) return e;
   for (int l = 1; l <= D; ++l) {
     Level& a = h->lev[l];
     Level& pa = h->lev[l - 1];
     const int nwarp = 8;
-    const size_t smem = m2l64 || !a.tri_m2l_hl
-                            ? sizeof(cplx) * ((size_t)a.P * (a.P + 1) + (size_t)nwarp * a.P)
-                            : sizeof(cplxf) * (2 * (size_t)a.P * (a.P + 1) + 2 * (size_t)nwarp * a.P);
-    const bool lists = smem > 200 * 1024;
+    const size_t smem = sizeof(cplx) * ((size_t)a.P * (a.P + 1) + (size_t)nwarp * a.P);
+    const bool lists = !m2l64 || smem > 200 * 1024;
     prof_begin(h, PH_LOCAL);
-    if (!lists && pa.tri_l2l_hl && !m2l64) {
+    if (grouped(l)) {
       e = k_tri_l2l_dd(h, l);
       if (e != cudaSuccess) return e;
     } else {
@@ -2461,32 +2495,17 @@ static cudaError_t matvec_tri_cached(pfmbem* h, const cplx* x, cplx* y) {
                                                        l == 1 ? 6 : 4, a.pidx);
     }
     prof_end(h, PH_LOCAL);
-    if (lists) continue;
+    if (lists || a.nchunk == 0) continue;
     prof_begin(h, PH_M2L);
-    if (a.tri_m2l_hl && !m2l64) {
-      e = k_tri_m2l_dd(h, l);
-      if (e != cudaSuccess) return e;
-    } else if (a.nchunk > 0) {
-      if (smem > 48 * 1024)
-        cudaFuncSetAttribute(m2l_offset_t_kernel<cplx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      m2l_offset_t_kernel<cplx><<<a.nchunk, 32 * nwarp, smem, st>>>(a.P, a.ch_off, a.ch_beg, a.ch_end, a.pr_tgt,
-                                                                     a.pr_src, a.pr_img, a.m2l, a.M, alpha, a.L);
-    }
+    if (smem > 48 * 1024)
+      cudaFuncSetAttribute(m2l_offset_t_kernel<cplx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    m2l_offset_t_kernel<cplx><<<a.nchunk, 32 * nwarp, smem, st>>>(a.P, a.ch_off, a.ch_beg, a.ch_end, a.pr_tgt,
+                                                                   a.pr_src, a.pr_img, a.m2l, a.M, alpha, a.L);
     prof_end(h, PH_M2L);
   }
   prof_begin(h, PH_L2P);
-  l2p_apply_t_kernel<cplx><<<leaf.nne, 256, 0, st>>>(leaf.ne, leaf.box_begin, leaf.box_end, leaf.P, E, h->l2p_c,
-                                                     leaf.L, h->U);
+  if ((e = k_tri_l2p(h, y)) != cudaSuccess) return e;
   prof_end(h, PH_L2P);
-  prof_begin(h, PH_NEAR);
-  near_apply_t_kernel<cplx><<<leaf.nne, 256, 0, st>>>(leaf.ne, leaf.box_begin, leaf.box_end, h->nc_base, h->nc_sbase,
-                                                      h->nc_src, h->nc_val, h->dens, h->U);
-  prof_end(h, PH_NEAR);
-  cplx c2{h->c2re, h->c2im};
-  prof_begin(h, PH_FIBER);
-  fiber_apply_t_kernel<cplx><<<h->nchunk, 256, 0, st>>>(h->fb_chunk, h->fib_off, h->fb_base, h->fb_val, h->o_pos,
-                                                        h->s_ph, c2, x, h->U, y, h->fb_circ);
-  prof_end(h, PH_FIBER);
   return cudaGetLastError();
 }
 

@@ -3318,120 +3318,352 @@ __global__ void split_hl_kernel(size_t n, const cplx* __restrict__ a, cplxf* __r
 // M2L of the triangle tree's offset groups (chunks of at most 16 pairs of one
 // offset) in double-float arithmetic: the FP64 result on the FP32 pipes, which
 // GB300 issues at 64 times its FP64 rate.  One block per chunk stages the
-// offset's operator as hi and lo parts ([P][P+1] each, padded rows); a warp per
-// pair splits its phased source multipole alpha^m M(src) into hi and lo, sums
-// each target coefficient with error-free products and sums (about 48 bits)
-// and adds it to L(tgt) in FP64.  L(tgt) holds the L2L part already.
-__global__ void tri_m2l_dd_kernel(int P, int noff, const int* __restrict__ chunk_off, const int* __restrict__ chunk_beg,
-                                  const int* __restrict__ chunk_end, const int* __restrict__ ptgt,
-                                  const int* __restrict__ psrc, const int* __restrict__ pimg,
-                                  const cplxf* __restrict__ Thl, const cplx* __restrict__ M, cplx alpha,
-                                  cplx* __restrict__ L) {
+// offset's operator as words of hi and lo parts (P = 2p + 1 is odd, so rows of P
+// words meet no bank twice); a warp takes two pairs at a time, so that each word
+// read serves both and four sums are in flight, splits their phased source
+// multipoles alpha^m M(src), sums each target coefficient with error-free products
+// and sums (about 48 bits) and adds it to L(tgt) in FP64.  FP32 instructions bound
+// it: 65 384 pairs at P = 61 are 10 GFP32 instructions a lane.
+template <int NP>
+__device__ __forceinline__ void tri_m2l_pairs(int P, int pi, const int* __restrict__ ptgt, const int* __restrict__ psrc,
+                                              const int* __restrict__ pimg, const float4* T, float4* wsm,
+                                              const cplx* __restrict__ M, cplx alpha, cplx* __restrict__ L, int lane) {
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < NP; ++q) {
+    const cplx ph = phase_m(alpha, pimg[pi + q]);
+    const cplx* Ms = M + (size_t)psrc[pi + q] * P;
+    for (int n = lane; n < P; n += 32) wsm[q * P + n] = dd_word(ph * Ms[n]);
+  }
+  __syncwarp();
+  for (int l = lane; l < P; l += 32) {
+    const float4* row = T + (size_t)l * P;
+    dflt re[NP], im[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) re[q] = im[q] = dflt{0, 0};
+#pragma unroll 2
+    for (int n = 0; n < P; ++n) {
+      const float4 t = row[n];
+#pragma unroll
+      for (int q = 0; q < NP; ++q) dd_cmac(re[q], im[q], t, wsm[q * P + n]);
+    }
+#pragma unroll
+    for (int q = 0; q < NP; ++q)
+      atomic_add(L + (size_t)ptgt[pi + q] * P + l, cplx{dd_value(re[q]), dd_value(im[q])});
+  }
+}
+
+// The levels of one launch: blocks first[i] .. first[i + 1] are the chunks of entry i.
+// All levels at once, for no level waits for another: launched one by one, each left a
+// last wave of its own (648, 372, 690, 966 and 1586 blocks on 456 resident).
+struct TriM2L {
+  int n;
+  int first[PF_MAXLEVEL + 1];
+  int P[PF_MAXLEVEL], noff[PF_MAXLEVEL];
+  const int *off[PF_MAXLEVEL], *beg[PF_MAXLEVEL], *end[PF_MAXLEVEL];
+  const int *tgt[PF_MAXLEVEL], *src[PF_MAXLEVEL], *img[PF_MAXLEVEL];
+  const cplxf* T[PF_MAXLEVEL];
+  const cplx* M[PF_MAXLEVEL];
+  cplx* L[PF_MAXLEVEL];
+};
+
+__global__ void __launch_bounds__(256, 3) tri_m2l_dd_kernel(const __grid_constant__ TriM2L a, cplx alpha) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  cplxf* sh = reinterpret_cast<cplxf*>(smraw);          // [P][P+1] hi
-  cplxf* sl = sh + (size_t)P * (P + 1);                  // [P][P+1] lo
-  cplxf* sm = sl + (size_t)P * (P + 1);                  // [warps][2][P] source hi, lo
-  const int o = chunk_off[blockIdx.x];
-  const int pb = chunk_beg[blockIdx.x], pe = chunk_end[blockIdx.x];
-  const size_t PP = (size_t)P * P;
-  const cplxf* Th = Thl + (size_t)o * PP;
-  const cplxf* Tl = Thl + (size_t)noff * PP + (size_t)o * PP;
-  for (int i = threadIdx.x; i < P * P; i += blockDim.x) {
-    const int r = i / P, c = i - r * P;
-    sh[r * (P + 1) + c] = Th[i];
-    sl[r * (P + 1) + c] = Tl[i];
+  float4* T = reinterpret_cast<float4*>(smraw);          // [P][P]
+  int i = 0;
+  while (i + 1 < a.n && (int)blockIdx.x >= a.first[i + 1]) ++i;
+  const int c = (int)blockIdx.x - a.first[i], P = a.P[i];
+  const int o = a.off[i][c], pb = a.beg[i][c], pe = a.end[i][c];
+  const int PP = P * P;
+  const cplxf* Th = a.T[i] + (size_t)o * PP;
+  const cplxf* Tl = Th + (size_t)a.noff[i] * PP;
+#pragma unroll 4
+  for (int q = threadIdx.x; q < PP; q += blockDim.x) {
+    const cplxf h = Th[q], l = Tl[q];
+    T[q] = make_float4(h.re, h.im, l.re, l.im);
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  cplxf* wh = sm + (size_t)warp * 2 * P;
-  cplxf* wl = wh + P;
+  float4* wsm = T + PP + (size_t)warp * 2 * P;           // the warp's two sources
   __syncthreads();
-  for (int pi = pb + warp; pi < pe; pi += nw) {
-    const int src = psrc[pi], tgt = ptgt[pi];
-    const cplx ph = phase_m(alpha, pimg[pi]);
-    __syncwarp();
-    for (int n = lane; n < P; n += 32) {
-      const cplx v = ph * M[(size_t)src * P + n];
-      wh[n] = cplxf{(float)v.re, (float)v.im};
-      wl[n] = split_lo(v);
-    }
-    __syncwarp();
-    for (int l = lane; l < P; l += 32) {
-      const cplxf* rh = sh + (size_t)l * (P + 1);
-      const cplxf* rl = sl + (size_t)l * (P + 1);
-      dflt re{0, 0}, im{0, 0};
-      for (int n = 0; n < P; ++n) dd_cmac(re, im, rh[n], rl[n], wh[n], wl[n]);
-      atomic_add(L + (size_t)tgt * P + l, cplx{dd_value(re), dd_value(im)});
-    }
+  for (int pi = pb + 2 * warp; pi < pe; pi += 2 * nw) {
+    if (pi + 1 < pe)
+      tri_m2l_pairs<2>(P, pi, a.tgt[i], a.src[i], a.img[i], T, wsm, a.M[i], alpha, a.L[i], lane);
+    else
+      tri_m2l_pairs<1>(P, pi, a.tgt[i], a.src[i], a.img[i], T, wsm, a.M[i], alpha, a.L[i], lane);
   }
 }
 
 // M2M and L2L of the triangle tree in double-float arithmetic, one block per
-// box and a thread per output coefficient; the operators' hi parts first, then
-// their lo parts (nop operators of [Pc][P] for M2M, [Pp][P] for L2L, rows of the
-// input coefficient, as the FP64 tables).  M2M: M(box) = sum over the non-empty
-// children ch (nch per box) of A_aidx[ch] M(ch).
-__global__ void tri_m2m_dd_kernel(const int* __restrict__ ne, int P, int Pc, int nop, const cplxf* __restrict__ Ahl,
-                                  const int* __restrict__ cbb, const int* __restrict__ cbe,
-                                  const cplx* __restrict__ Mc, cplx* __restrict__ Mp, int nch,
-                                  const int* __restrict__ aidx) {
+// box; the operators' hi parts first, then their lo parts (nop operators of
+// [Pc][P] for M2M, [Pp][P] for L2L, rows of the input coefficient, as the FP64
+// tables).  A column of threads per output coefficient shares its sum, and the
+// shares meet in shared memory: with one thread per coefficient a box was one
+// chain over all children (296 us of M2M and 129 us of L2L in a product on 16384
+// elements at p = 30).
+// M2M: M(box) = sum over the non-empty children ch (nch per box) of A_aidx[ch] M(ch),
+// share y of the column taking every G-th coefficient of every child; it also clears
+// L(box) for the M2L's sums.
+constexpr int TRI_Y = 16;
+__global__ void __launch_bounds__(1024) tri_m2m_dd_kernel(const int* __restrict__ ne, int P, int Pc, int nop,
+                                                          const cplxf* __restrict__ Ahl, const int* __restrict__ cbb,
+                                                          const int* __restrict__ cbe, const cplx* __restrict__ Mc,
+                                                          cplx* __restrict__ Mp, int nch, const int* __restrict__ aidx,
+                                                          cplx* __restrict__ Lz) {
+  extern __shared__ float4 tri_sm[];
   const int box = ne[blockIdx.x];
-  __shared__ cplxf sh[PF_NCOEF], sl[PF_NCOEF];
+  const int n = threadIdx.x, G = blockDim.y;
+  float4* sw = tri_sm;                     // [nch][Pc] the children's multipoles
   const size_t lo = (size_t)nop * Pc * P;
-  dflt re{0, 0}, im{0, 0};
-  for (int q = 0; q < nch; ++q) {
-    const int ch = nch * box + q;
-    if (cbb[ch] >= cbe[ch]) continue;   // empty child (uniform across the block)
-    __syncthreads();
-    for (int i = threadIdx.x; i < Pc; i += blockDim.x) {
-      const cplx v = Mc[(size_t)ch * Pc + i];
-      sh[i] = cplxf{(float)v.re, (float)v.im};
-      sl[i] = split_lo(v);
-    }
-    __syncthreads();
-    if (threadIdx.x < P) {
-      const cplxf* ah = Ahl + (size_t)aidx[ch] * Pc * P + threadIdx.x;
-      for (int m = 0; m < Pc; ++m) dd_cmac(re, im, ah[(size_t)m * P], ah[lo + (size_t)m * P], sh[m], sl[m]);
-    }
+  for (int i = threadIdx.y * blockDim.x + n; i < nch * Pc; i += G * blockDim.x) {
+    const int q = i / Pc, ch = nch * box + q;
+    if (cbb[ch] < cbe[ch]) sw[i] = dd_word(Mc[(size_t)nch * box * Pc + i]);
   }
-  if (threadIdx.x < P) Mp[(size_t)box * P + threadIdx.x] = cplx{dd_value(re), dd_value(im)};
+  __syncthreads();
+  dflt re{0, 0}, im{0, 0};
+  if (n < P)
+    for (int q = 0; q < nch; ++q) {
+      const int ch = nch * box + q;
+      if (cbb[ch] >= cbe[ch]) continue;
+      const cplxf* ah = Ahl + (size_t)aidx[ch] * Pc * P + n;
+#pragma unroll 4
+      for (int m = threadIdx.y; m < Pc; m += G) {
+        const cplxf h = ah[(size_t)m * P], l = ah[lo + (size_t)m * P];
+        dd_cmac(re, im, make_float4(h.re, h.im, l.re, l.im), sw[q * Pc + m]);
+      }
+    }
+  __syncthreads();
+  if (n < P) tri_sm[threadIdx.y * P + n] = make_float4(re.h, im.h, re.l, im.l);
+  __syncthreads();
+  if (threadIdx.y == 0 && n < P) {
+    for (int q = 1; q < G; ++q) {
+      const float4 w = tri_sm[q * P + n];
+      re = dd_add(re, dflt{w.x, w.z});
+      im = dd_add(im, dflt{w.y, w.w});
+    }
+    Mp[(size_t)box * P + n] = cplx{dd_value(re), dd_value(im)};
+    Lz[(size_t)box * P + n] = cplx{0, 0};
+  }
 }
 
-// L2L: L(box) = B_pidx[box] L(parent), the parent box / nchp.
-__global__ void tri_l2l_dd_kernel(const int* __restrict__ ne, int P, int Pp, int nop, const cplxf* __restrict__ Bhl,
+// L2L: L(box) += B_pidx[box] L(parent), the parent box / nchp.
+__global__ void __launch_bounds__(1024) tri_l2l_dd_kernel(const int* __restrict__ ne, int P, int Pp, int nop, const cplxf* __restrict__ Bhl,
                                   const cplx* __restrict__ Lp, cplx* __restrict__ L, int nchp,
                                   const int* __restrict__ pidx) {
   const int box = ne[blockIdx.x];
-  __shared__ cplxf sh[PF_NCOEF], sl[PF_NCOEF];
+  const int n = threadIdx.x, G = blockDim.y;
+  extern __shared__ float4 tri_sm[];
+  float4 *sw = tri_sm, *sr = tri_sm + Pp;  // [Pp] the parent's expansion, [G][P] the shares
   const int par = box / nchp;
-  for (int i = threadIdx.x; i < Pp; i += blockDim.x) {
-    const cplx v = Lp[(size_t)par * Pp + i];
-    sh[i] = cplxf{(float)v.re, (float)v.im};
-    sl[i] = split_lo(v);
+  for (int i = threadIdx.y * blockDim.x + n; i < Pp; i += G * blockDim.x) sw[i] = dd_word(Lp[(size_t)par * Pp + i]);
+  __syncthreads();
+  dflt re{0, 0}, im{0, 0};
+  if (n < P) {
+    const size_t lo = (size_t)nop * Pp * P;
+    const cplxf* bh = Bhl + (size_t)pidx[box] * Pp * P + n;
+#pragma unroll 4
+    for (int m = threadIdx.y; m < Pp; m += G) {
+      const cplxf h = bh[(size_t)m * P], l = bh[lo + (size_t)m * P];
+      dd_cmac(re, im, make_float4(h.re, h.im, l.re, l.im), sw[m]);
+    }
+    sr[threadIdx.y * P + n] = make_float4(re.h, im.h, re.l, im.l);
   }
   __syncthreads();
-  if (threadIdx.x < P) {
-    const size_t lo = (size_t)nop * Pp * P;
-    const cplxf* bh = Bhl + (size_t)pidx[box] * Pp * P + threadIdx.x;
-    dflt re{0, 0}, im{0, 0};
-    for (int m = 0; m < Pp; ++m) dd_cmac(re, im, bh[(size_t)m * P], bh[lo + (size_t)m * P], sh[m], sl[m]);
-    L[(size_t)box * P + threadIdx.x] = cplx{dd_value(re), dd_value(im)};
+  if (threadIdx.y == 0 && n < P) {
+    for (int q = 1; q < G; ++q) {
+      const float4 w = sr[q * P + n];
+      re = dd_add(re, dflt{w.x, w.z});
+      im = dd_add(im, dflt{w.y, w.w});
+    }
+    cplx* o = L + (size_t)box * P + n;
+    *o += cplx{dd_value(re), dd_value(im)};
   }
+}
+
+// Threads over the coefficients by shares of a column: short chains on levels of few
+// boxes (below eight blocks of 256 threads per SM), a block of four shares elsewhere.
+static dim3 tri_block(int P, int nbox) {
+  const int x = ((P + 31) / 32) * 32;
+  return dim3(x, std::max(1, std::min(nbox < 8 * 152 ? TRI_Y : 4, 1024 / x)));
+}
+
+// ------------------------------------- triangle tree: tables as double-float words
+// n FP64 values turned into the words of their hi and lo parts where they lie.
+__global__ void dd_words_kernel(size_t n, cplx* a) {
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const cplx v = a[i];
+    reinterpret_cast<float4*>(a)[i] = dd_word(v);
+  }
+}
+
+// The operator between the cells, L0 = TOP M0 (the words of TOP [rows][rows]): one
+// warp per row, the multipoles as words in shared memory, a tile of TRI_TILE at a
+// time.  Bound by the read of TOP; in FP64 instructions their pipe bound it (213 us
+// for 3904 rows, 244 MB).
+constexpr int TRI_TILE = 1024;
+__global__ void __launch_bounds__(256) tri_top_kernel(int rows, const float4* __restrict__ TOP,
+                                                      const cplx* __restrict__ M0, cplx* __restrict__ L0) {
+  __shared__ float4 sw[TRI_TILE];
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const float4* t = TOP + (size_t)min(row, rows - 1) * rows;
+  dflt re{0, 0}, im{0, 0};
+  for (int c0 = 0; c0 < rows; c0 += TRI_TILE) {
+    const int nc = min(TRI_TILE, rows - c0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nc; i += 256) sw[i] = dd_word(M0[c0 + i]);
+    __syncthreads();
+#pragma unroll 4
+    for (int i = lane; i < nc; i += 32) dd_cmac(re, im, __ldcs(t + c0 + i), sw[i]);
+  }
+  const dflt r = dd_wsum(re), q = dd_wsum(im);
+  if (lane == 0 && row < rows) L0[row] = cplx{dd_value(r), dd_value(q)};
+}
+
+// Same-fiber rows of the triangle tree's cached product, y = B x by chunks of rows of a
+// fiber (chunk: fiber, first and last row).  A circulant fiber's generating row pair
+// and x are staged as words and a warp sums a row pair with x rotated by 2e, sum_c
+// R[(c - 2e) mod 2N] x[c] = sum_c R[c] x[(c + 2e) mod 2N]; the rows of another fiber
+// are FP64 sums over its table (converting a word costs what it saves there).  FP64
+// sums and the division by the phase in one lane kept the FP64 pipe busy for 299 us
+// at 64 circulant fibers of 256 elements.
+__global__ void __launch_bounds__(256) tri_fiber_kernel(const int* __restrict__ chunk, const int* __restrict__ foff,
+                                                        const int64_t* __restrict__ fbase,
+                                                        const cplx* __restrict__ val, const cplx* __restrict__ x,
+                                                        cplx* __restrict__ y, const int* __restrict__ circ) {
+  extern __shared__ float4 tri_sm[];
+  const int fb = chunk[3 * blockIdx.x], rb = chunk[3 * blockIdx.x + 1], re = chunk[3 * blockIdx.x + 2];
+  const int f0 = foff[fb], n2 = 2 * (foff[fb + 1] - f0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const cplx* B = val + fbase[fb];
+  if (circ[fb]) {
+    float4 *xw = tri_sm, *rw = tri_sm + n2;              // x, the row pair
+    for (int i = threadIdx.x; i < n2; i += blockDim.x) xw[i] = dd_word(x[2 * f0 + i]);
+    for (int i = threadIdx.x; i < 2 * n2; i += blockDim.x) rw[i] = dd_word(B[i]);
+    __syncthreads();
+    for (int r = rb + 2 * warp; r < re; r += 2 * nw) {   // chunks hold whole row pairs
+      dflt a{0, 0}, b{0, 0}, c{0, 0}, d{0, 0};
+#pragma unroll 2
+      for (int i = lane; i < n2; i += 32) {
+        int j = i + r;
+        if (j >= n2) j -= n2;
+        const float4 v = xw[j];
+        dd_cmac(a, b, rw[i], v);
+        dd_cmac(c, d, rw[n2 + i], v);
+      }
+      const dflt s = dd_wsum4(a, b, c, d, lane);         // lanes 0, 8, 16, 24
+      if ((lane & 7) == 0) reinterpret_cast<double*>(y + 2 * f0 + r)[lane >> 3] = dd_value(s);
+    }
+    return;
+  }
+  cplx* xs = reinterpret_cast<cplx*>(tri_sm);
+  for (int i = threadIdx.x; i < n2; i += blockDim.x) xs[i] = x[2 * f0 + i];
+  __syncthreads();
+  for (int r = rb + warp; r < re; r += nw) {
+    const cplx* row = B + (int64_t)r * n2;
+    cplx a{0, 0}, b{0, 0};
+    int c = lane;
+    for (; c + 32 < n2; c += 64) {
+      const cplx r0 = row[c], r1 = row[c + 32];
+      a += r0 * xs[c];
+      b += r1 * xs[c + 32];
+    }
+    if (c < n2) a += row[c] * xs[c];
+    a = wsum(a + b);
+    if (lane == 0) y[2 * f0 + r] = a;
+  }
+}
+
+// L2P and the near sums (U, already there), added to y in the caller's order:
+// y_e += alpha^{m0} (U + U', c2 (dU + dU')), U'_s = sum_l c[s][0][l] L_l, dU'_s =
+// sum_l c[s][1][l] L_l with the words of c.  One block per leaf, 16 elements by 16
+// shares of the coefficients: the words lie element by element (entry (q, l) of
+// element s at (q P + l) E + s), so the elements of a leaf are read together.
+__global__ void __launch_bounds__(256) tri_l2p_add_kernel(
+    const int* __restrict__ ne, const int* __restrict__ bb, const int* __restrict__ be, int P, int E,
+    const float4* __restrict__ coef, const cplx* __restrict__ L, const cplx* __restrict__ U,
+    const int* __restrict__ perm, const cplx* __restrict__ sph, cplx c2, cplx* __restrict__ y) {
+  __shared__ float4 sL[PF_NCOEF], red[2][16][17];
+  const int box = ne[blockIdx.x], el = threadIdx.x & 15, sl = threadIdx.x >> 4;
+  for (int l = threadIdx.x; l < P; l += 256) sL[l] = dd_word(L[(size_t)box * P + l]);
+  for (int s0 = bb[box]; s0 < be[box]; s0 += 16) {
+    const int s = s0 + el;
+    __syncthreads();
+    dflt a{0, 0}, b{0, 0}, c{0, 0}, d{0, 0};
+    if (s < be[box])
+#pragma unroll 4
+      for (int l = sl; l < P; l += 16) {
+        const float4 v = sL[l];
+        dd_cmac(a, b, coef[(size_t)l * E + s], v);
+        dd_cmac(c, d, coef[(size_t)(P + l) * E + s], v);
+      }
+    red[0][sl][el] = make_float4(a.h, b.h, a.l, b.l);
+    red[1][sl][el] = make_float4(c.h, d.h, c.l, d.l);
+    __syncthreads();
+    if (sl < 2 && s < be[box]) {
+      dflt u{0, 0}, v{0, 0};
+      for (int q = 0; q < 16; ++q) {
+        const float4 w = red[sl][q][el];
+        u = dd_add(u, dflt{w.x, w.z});
+        v = dd_add(v, dflt{w.y, w.w});
+      }
+      const cplx t = conj(sph[s]) * (U[2 * s + sl] + cplx{dd_value(u), dd_value(v)});   // |sph| = 1
+      y[2 * perm[s] + sl] += sl ? c2 * t : t;
+    }
+  }
+}
+
+// TOP and the L2P coefficients as words (once, at the end of the set-up).
+cudaError_t k_tri_words(pfmbem* h) {
+  const size_t rows = (size_t)h->nroot * h->lev[0].P, nc = (size_t)h->E * 2 * h->lev[h->D].P;
+  dd_words_kernel<<<(unsigned)std::min<size_t>((rows * rows + 255) / 256, 8192), 256, 0, h->stream>>>(rows * rows,
+                                                                                                     h->root);
+  dd_words_kernel<<<(unsigned)std::min<size_t>((nc + 255) / 256, 8192), 256, 0, h->stream>>>(nc, h->l2p_c);
+  return cudaGetLastError();
+}
+
+cudaError_t k_tri_top(pfmbem* h, cudaStream_t st) {
+  const int rows = h->nroot * h->lev[0].P;
+  tri_top_kernel<<<(rows + 7) / 8, 256, 0, st>>>(rows, reinterpret_cast<const float4*>(h->root), h->lev[0].M,
+                                                 h->lev[0].L);
+  return cudaGetLastError();
+}
+
+cudaError_t k_tri_fiber(pfmbem* h, const cplx* x, cplx* y, cudaStream_t st) {
+  const size_t smem = sizeof(float4) * 3 * 2 * (size_t)h->max_fiber;
+  if (smem > 48 * 1024) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(tri_fiber_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  tri_fiber_kernel<<<h->nchunk, 256, smem, st>>>(h->fb_chunk, h->fib_off, h->fb_base, h->fb_val, x, y, h->fb_circ);
+  return cudaGetLastError();
+}
+
+cudaError_t k_tri_l2p(pfmbem* h, cplx* y) {
+  const Level& leaf = h->lev[h->D];
+  tri_l2p_add_kernel<<<leaf.nne, 256, 0, h->stream>>>(leaf.ne, leaf.box_begin, leaf.box_end, leaf.P, h->E,
+                                                      reinterpret_cast<const float4*>(h->l2p_c), leaf.L, h->U,
+                                                      h->s_perm, h->s_ph, cplx{h->c2re, h->c2im}, y);
+  return cudaGetLastError();
 }
 
 cudaError_t k_tri_m2m_dd(pfmbem* h, int l) {
   const Level& a = h->lev[l];
   const Level& c = h->lev[l + 1];
-  tri_m2m_dd_kernel<<<a.nne, ((a.P + 31) / 32) * 32, 0, h->stream>>>(a.ne, a.P, c.P, a.tri_nop, a.tri_m2m_hl,
-                                                                     c.box_begin, c.box_end, c.M, a.M,
-                                                                     l == 0 ? 6 : 4, c.pidx);
+  const int nch = l == 0 ? 6 : 4;
+  const dim3 nt = tri_block(a.P, a.nne);
+  const size_t smem = sizeof(float4) * std::max((size_t)nch * c.P, (size_t)nt.y * a.P);
+  tri_m2m_dd_kernel<<<a.nne, nt, smem, h->stream>>>(a.ne, a.P, c.P, a.tri_nop, a.tri_m2m_hl, c.box_begin, c.box_end,
+                                                    c.M, a.M, nch, c.pidx, a.L);
   return cudaGetLastError();
 }
 
 cudaError_t k_tri_l2l_dd(pfmbem* h, int l) {
   const Level& a = h->lev[l];
   const Level& pa = h->lev[l - 1];
-  tri_l2l_dd_kernel<<<a.nne, ((a.P + 31) / 32) * 32, 0, h->stream>>>(a.ne, a.P, pa.P, pa.tri_nop, pa.tri_l2l_hl,
-                                                                     pa.L, a.L, l == 1 ? 6 : 4, a.pidx);
+  const dim3 nt = tri_block(a.P, a.nne);
+  const size_t smem = sizeof(float4) * ((size_t)pa.P + (size_t)nt.y * a.P);
+  tri_l2l_dd_kernel<<<a.nne, nt, smem, h->stream>>>(a.ne, a.P, pa.P, pa.tri_nop, pa.tri_l2l_hl, pa.L, a.L,
+                                                    l == 1 ? 6 : 4, a.pidx);
   return cudaGetLastError();
 }
 
@@ -3453,24 +3685,36 @@ cudaError_t k_tri_m2l_split(pfmbem* h, int l) {
   return cudaGetLastError();
 }
 
-// Level l's M2L by offset groups in double-float arithmetic (after its L2L).
-cudaError_t k_tri_m2l_dd(pfmbem* h, int l) {
-  const Level& L = h->lev[l];
-  if (L.nchunk == 0) return cudaSuccess;
-  const int nwarp = 8;
-  const size_t smem = sizeof(cplxf) * (2 * (size_t)L.P * (L.P + 1) + 2 * (size_t)nwarp * L.P);
+// Shared memory of a level's M2L: the operator and two sources for each of eight warps.
+size_t k_tri_m2l_smem(int P) { return sizeof(float4) * ((size_t)P * P + 2 * 8 * (size_t)P); }
+
+// M2L by offset groups in double-float arithmetic, added to L (which the upward pass
+// cleared), of every level whose operators fit shared memory.
+cudaError_t k_tri_m2l_dd(pfmbem* h) {
+  TriM2L a{};
+  size_t smem = 0;
+  for (int l = h->D; l >= 1; --l) {
+    const Level& L = h->lev[l];
+    if (L.nchunk == 0 || k_tri_m2l_smem(L.P) > TRI_M2L_SMEM) continue;
+    const int i = a.n++;
+    a.first[i + 1] = a.first[i] + L.nchunk;
+    a.P[i] = L.P;
+    a.noff[i] = L.tri_noff;
+    a.off[i] = L.ch_off; a.beg[i] = L.ch_beg; a.end[i] = L.ch_end;
+    a.tgt[i] = L.pr_tgt; a.src[i] = L.pr_src; a.img[i] = L.pr_img;
+    a.T[i] = L.tri_m2l_hl;
+    a.M[i] = L.M;
+    a.L[i] = L.L;
+    smem = std::max(smem, k_tri_m2l_smem(L.P));
+  }
+  if (a.n == 0) return cudaSuccess;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(tri_m2l_dd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  tri_m2l_dd_kernel<<<L.nchunk, 32 * nwarp, smem, h->stream>>>(L.P, L.tri_noff, L.ch_off, L.ch_beg, L.ch_end,
-                                                                L.pr_tgt, L.pr_src, L.pr_img, L.tri_m2l_hl, L.M,
-                                                                h->alpha, L.L);
+  tri_m2l_dd_kernel<<<a.first[a.n], 256, smem, h->stream>>>(a, h->alpha);
   return cudaGetLastError();
 }
-
-namespace {
-}  // namespace
 
 // The top operators of the fused product on stream st: R T_0 (root fold) and,
 // with level 3 present, T_1 T_2 and R T_0 T_1 T_2; st must be ordered after the

@@ -633,8 +633,14 @@ static pfmbem_status build_plan_tri(pfmbem* h, const double* nodes, const std::v
                     l < D ? sh_v[l] : nullptr, l < D ? (int)sh_off[l].v.size() : 0));
   CK(k_wide_top(h, dv, S, X, nbr_dev));
   if (h->tri_cache) {
+    // the product's second chain (matvec_tri_cached)
+    if (!h->aux[0]) CK(pool_stream(h->dev, &h->aux[0]));
+    if (!h->aux_ev[0]) CK(pool_event(h->dev, &h->aux_ev[0]));
+    if (!h->fork_ev) CK(pool_event(h->dev, &h->fork_ev));
+    if (!h->side_ev) CK(pool_event(h->dev, &h->side_ev));
     CK(k_tri_caches(h));
     for (int l = 0; l <= D; ++l) CK(k_tri_m2l_split(h, l));
+    CK(k_tri_words(h));
   }
   h->ub_on = false;
   pin_release_async(h);
