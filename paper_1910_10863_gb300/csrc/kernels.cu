@@ -930,6 +930,7 @@ __global__ void p2m_f64_kernel(const int* __restrict__ ne, const int* __restrict
                                const double2* __restrict__ ctr) {
   const int box = ne[blockIdx.x];
   const int P = 2 * p + 1;
+  const size_t row = wgt ? box : blockIdx.x;      // no weights: unscaled, a row per listed box
   __shared__ double acc[2 * PF_NCOEF];
   for (int i = threadIdx.x; i < 2 * P; i += blockDim.x) acc[i] = 0.0;
   __syncthreads();
@@ -967,13 +968,13 @@ __global__ void p2m_f64_kernel(const int* __restrict__ ne, const int* __restrict
     cplx nuc{nu.x, nu.y};
     for (int n = -p; n <= p; ++n) {
       cplx v = a * (conj(nuc) * Jm[p + n] - nuc * Jm[p + n + 2]) + bcoef * Jm[p + n + 1];
-      double iw = 1.0 / wgt[n + p];
+      double iw = wgt ? 1.0 / wgt[n + p] : 1.0;
       atomicAdd(&acc[2 * (n + p)], v.re * iw);
       atomicAdd(&acc[2 * (n + p) + 1], v.im * iw);
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < P; i += blockDim.x) Mout[(size_t)box * P + i] = cplx{acc[2 * i], acc[2 * i + 1]};
+  for (int i = threadIdx.x; i < P; i += blockDim.x) Mout[row * P + i] = cplx{acc[2 * i], acc[2 * i + 1]};
 }
 
 // ---------------------------------------------------------------- M2M (FP64)
@@ -2871,33 +2872,34 @@ struct FieldTree {
   const double2* ctr[PF_MAXLEVEL + 1]; // box centres (triangle tree), null: from the Morton code
 };
 
-// x1-derivative of sum_n w_n M_n H^+_n(k v)
-__device__ __forceinline__ cplx multipole_dx1(double k, double vx, double vy, int p, const double* __restrict__ w,
-                                              const cplx* __restrict__ M) {
+// sum_{|n| <= q} c_n H^+_n(k v) (WU) and its x1-derivative (WD), c_n = w_n M_n, or M_n
+// without weights; q <= p, the order of M.
+template <bool WU, bool WD>
+__device__ __forceinline__ void multipole_eval(double k, double vx, double vy, int p, int q,
+                                               const double* __restrict__ w, const cplx* __restrict__ M, cplx& u,
+                                               cplx& d) {
   const double r2 = vx * vx + vy * vy, ir = rsqrt(r2), x = k * r2 * ir;
   const cplx z{vx * ir, vy * ir};
   double J0, J1, Y0, Y1;
   bessel01(x, J0, J1, Y0, Y1);
   cplx hm{J0, Y0}, h{J1, Y1}, zp{1, 0};
   const double ix2 = 2.0 / x;
-  // coefficients c_n = w_n M_n around +-n: a_n = c_n, b_n = c_-n
-  const cplx c0 = w[p] * M[p];
-  cplx am = c0, a{0, 0}, b = c0, bn{0, 0};    // am = c_{n-1}, a = c_n, b = c_{-(n-1)}, bn = c_{-n}
-  if (p >= 1) {
-    a = w[p + 1] * M[p + 1];
-    bn = w[p - 1] * M[p - 1];
-  }
-  cplx d = hm * (a - bn);                      // m = 0: c_1 - c_-1
+  auto coef = [&](int n) -> cplx {
+    if (n > q || n < -q) return cplx{0, 0};
+    return w ? w[p + n] * M[p + n] : M[p + n];
+  };
+  // coefficients around +-n: a_n = c_n, b_n = c_-n
+  const cplx c0 = coef(0);
+  cplx am = c0, a = coef(1), b = c0, bn = coef(-1);    // am = c_{n-1}, a = c_n, b = c_{-(n-1)}, bn = c_{-n}
+  if (WU) u = hm * c0;
+  if (WD) d = hm * (a - bn);                   // m = 0: c_1 - c_-1
   double sg = -1.0;
-  for (int n = 1; n <= p + 1; ++n) {
+  for (int n = 1; n <= q + (WD ? 1 : 0); ++n) {
     zp = zp * z;
     const cplx hp = h * zp, hn = sg * (h * conj(zp));   // H^+_n, H^+_-n
-    cplx a2{0, 0}, b2{0, 0};                             // c_{n+1}, c_{-(n+1)}
-    if (n + 1 <= p) {
-      a2 = w[p + n + 1] * M[p + n + 1];
-      b2 = w[p - n - 1] * M[p - n - 1];
-    }
-    d += hp * (a2 - am) + hn * (b - b2);
+    const cplx a2 = coef(n + 1), b2 = coef(-n - 1);      // c_{n+1}, c_{-(n+1)}
+    if (WU) u += hp * a + hn * bn;
+    if (WD) d += hp * (a2 - am) + hn * (b - b2);
     am = a;
     a = a2;
     b = bn;
@@ -2907,7 +2909,7 @@ __device__ __forceinline__ cplx multipole_dx1(double k, double vx, double vy, in
     hm = h;
     h = hnext;
   }
-  return (0.5 * k) * d;
+  if (WD) d = (0.5 * k) * d;
 }
 
 __global__ void __launch_bounds__(FT_NT) field_tree_kernel(
@@ -2946,8 +2948,10 @@ __global__ void __launch_bounds__(FT_NT) field_tree_kernel(
       }
       const double vx = x.x - cx, vy = x.y - (cy + m * H);
       if (vx * vx + vy * vy >= ft.far2[l]) {
-        dacc += ipow_phase(alpha, m) *
-                multipole_dx1(k, vx, vy, ft.p[l], ft.w[l], ft.M[l] + (size_t)box * (2 * ft.p[l] + 1));
+        cplx u, du;
+        multipole_eval<false, true>(k, vx, vy, ft.p[l], ft.p[l], ft.w[l],
+                                    ft.M[l] + (size_t)box * (2 * ft.p[l] + 1), u, du);
+        dacc += ipow_phase(alpha, m) * du;
       } else {
         const int o = atomicAdd(&s_n[cur], 1);
         if (o < FT_CAP) {
@@ -2997,6 +3001,192 @@ __global__ void __launch_bounds__(FT_NT) field_tree_kernel(
     part[4 * (size_t)pi] = cplx{0, 0};
     part[4 * (size_t)pi + 1] = dacc;
   }
+}
+
+// u and its x1-derivative through the multipoles of the leaves, of the same quadrature
+// as the direct sum.  Where a density radiates almost nothing u cancels to 1e-6 of its
+// terms and the Gauss ladder's remainders (1e-14 of an element's term) show, so a leaf
+// enters as a whole only where the ladder gives all its elements one rule g = 2, 3 or 4
+// (54 h <= r for g = 3, 790 h for 2; other leaves, and those nearer than the expansion
+// allows, go element by element), by the multipoles of that rule's nodes, taken once per
+// call (field_rules).  The expansion ends where its remainder is below 10^-15 of the
+// leaf's field: at order q with (R / r)^q and (k R / 2)^q / q! below it.
+// A block takes slice sl of nsl of a point's (leaf, image) pairs; the pairs that go by
+// elements are collected in shared memory and summed together when the list fills.
+// Bound by the FP64 pipe: some 500 instructions a leaf, against 500 to 700 an element.
+// 1024 points on 16384 elements: 8.0 ms, 64 ms element by element.
+constexpr int FL_NT = 256, FL_CAP = 1024;
+struct FieldLeaf {
+  int nleaf, D, p, nmin;                 // nmin: order from which (k R / 2)^n / n! is below 1e-16
+  double d, R, far2;                     // leaf side, radius, squared distance from which a leaf is far
+  const int *ne, *bb, *be;
+  const double2* ctr;
+  const double2* hr;                     // [nleaf] shortest and longest element
+  const cplx* M;                         // [3][nleaf][2p+1] multipoles of the rules 2, 3, 4
+};
+
+__global__ void leaf_lengths_kernel(int nleaf, const int* __restrict__ ne, const int* __restrict__ bb,
+                                    const int* __restrict__ be, const double* __restrict__ sh,
+                                    double2* __restrict__ hr) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nleaf) return;
+  double lo = 1e300, hi = 0;
+  for (int f = bb[ne[i]]; f < be[ne[i]]; ++f) {
+    lo = fmin(lo, sh[f]);
+    hi = fmax(hi, sh[f]);
+  }
+  hr[i] = double2{lo, hi};
+}
+
+template <bool WU, bool WD>
+__global__ void __launch_bounds__(FL_NT) field_leaf_kernel(
+    const __grid_constant__ FieldLeaf fl, int npts, const double2* __restrict__ pts, int nsl, double k, double eta,
+    double H, double ox, double oy, double x0, double y0, int mdir, cplx alpha, const double2* __restrict__ sc,
+    const double2* __restrict__ st, const double2* __restrict__ snu, const double* __restrict__ sh,
+    const cplx* __restrict__ dens, int p0, const double* __restrict__ w0, const cplx* __restrict__ L0,
+    cplx* __restrict__ part) {
+  if ((int)blockIdx.x >= npts * nsl) {
+    local_part(((int)blockIdx.x - npts * nsl) * FL_NT + threadIdx.x, npts, pts, nsl, k, H, ox, oy, y0, p0, w0, L0,
+               part);
+    return;
+  }
+  __shared__ int s_li[FL_CAP], s_img[FL_CAP], s_off[FL_CAP + 1], s_n;
+  __shared__ cplx s_red[2][FL_NT / 32];
+  const int tid = threadIdx.x, lane = tid & 31, pi = blockIdx.x / nsl, sl = blockIdx.x - pi * nsl;
+  const int nim = 2 * mdir + 1, jobs = fl.nleaf * nim, P = 2 * fl.p + 1;
+  double2 x = pts[pi];
+  x.y -= floor((x.y - y0) / H) * H;
+  cplx acc{0, 0}, dacc{0, 0};
+  if (tid == 0) s_n = 0;
+  __syncthreads();
+  for (int base = sl * FL_NT; base < jobs; base += nsl * FL_NT) {
+    const int t = base + tid;
+    if (t < jobs) {
+      const int li = t / nim, m = t - li * nim - mdir, box = fl.ne[li];
+      double cx, cy;
+      if (fl.ctr) {
+        cx = fl.ctr[box].x;
+        cy = fl.ctr[box].y;
+      } else {
+        morton_centre(box, fl.D, fl.d, x0, y0, cx, cy);
+      }
+      const double vx = x.x - cx, vy = x.y - (cy + m * H), r2 = vx * vx + vy * vy;
+      const double2 hr = fl.hr[li];
+      const double r = sqrt(r2), lo = (r - fl.R) * (1.0 - 1e-12), hi = (r + fl.R) * (1.0 + 1e-12);
+      int g = 0;
+      if (r2 >= fl.far2)
+        for (int q = 2; q <= 4; ++q)
+          if (lo >= c_glthr[0][q] * hr.y && hi < c_glthr[0][q - 1] * hr.x) g = q;
+      if (g) {
+        const int q = (int)ceilf(15.2f / log10f((float)(r / (fl.R + 0.5 * hr.y))));
+        cplx u, du;
+        multipole_eval<WU, WD>(k, vx, vy, fl.p, min(fl.p, max(fl.nmin, q)), nullptr,
+                               fl.M + ((size_t)(g - 2) * fl.nleaf + li) * P, u, du);
+        const cplx ph = ipow_phase(alpha, m);
+        if (WU) acc += ph * u;
+        if (WD) dacc += ph * du;
+      } else {
+        const int o = atomicAdd(&s_n, 1);          // below FL_CAP: a list of more than FL_CAP - FL_NT was emptied
+        s_li[o] = li;
+        s_img[o] = m;
+      }
+    }
+    __syncthreads();
+    const int nl = s_n;
+    if (nl > 0 && (nl > FL_CAP - FL_NT || base + nsl * FL_NT >= jobs)) {
+      if (tid < 32) {                              // first element of every entry
+        int run = 0;
+        for (int i0 = 0; i0 < nl; i0 += 32) {
+          const int i = i0 + lane, box = i < nl ? fl.ne[s_li[i]] : 0;
+          const int c = i < nl ? fl.be[box] - fl.bb[box] : 0;
+          int v = c;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int n = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += n;
+          }
+          if (i < nl) s_off[i] = run + v - c;
+          run += __shfl_sync(0xffffffffu, v, 31);
+        }
+        if (lane == 0) s_off[nl] = run;
+      }
+      __syncthreads();
+      const double2 nx{1.0, 0.0};
+      for (int e = tid; e < s_off[nl]; e += FL_NT) {
+        int lo = 0, hi = nl - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (s_off[mid] <= e) lo = mid;
+          else hi = mid - 1;
+        }
+        const int f = fl.bb[fl.ne[s_li[lo]]] + e - s_off[lo], m = s_img[lo];
+        double2 c = sc[f];
+        c.y += m * H;
+        const double hh = sh[f];
+        const double q = sqrt((x.x - c.x) * (x.x - c.x) + (x.y - c.y) * (x.y - c.y)) / hh;
+        cplx S{0, 0}, Dv{0, 0}, K{0, 0}, T{0, 0};
+        pair4_f64(k, x, nx, c, st[f], snu[f], hh, gl_order(q, 0), S, Dv, K, T);
+        const cplx ph = ipow_phase(alpha, m);
+        if (WU) acc += ph * (Dv * dens[2 * f] - eta * mul_i(S * dens[2 * f + 1]));
+        if (WD) dacc += ph * (T * dens[2 * f] - eta * mul_i(K * dens[2 * f + 1]));
+      }
+      __syncthreads();
+      if (tid == 0) s_n = 0;
+    }
+    __syncthreads();
+  }
+  if (WU) acc = warp_sum(acc);
+  if (WD) dacc = warp_sum(dacc);
+  if (lane == 0) {
+    s_red[0][tid >> 5] = acc;
+    s_red[1][tid >> 5] = dacc;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int i = 1; i < FL_NT / 32; ++i) {
+      acc += s_red[0][i];
+      dacc += s_red[1][i];
+    }
+    cplx* o = part + 2 * ((size_t)pi * (nsl + 1) + sl);
+    o[0] = acc;
+    o[1] = dacc;
+  }
+}
+
+// Whether the field goes by leaves: orders of the default rule and elements of at most a
+// quarter of a leaf, as in field_tree, and points enough to pay for three rules'
+// multipoles (nine nodes an element, the work of about seven points' direct sums).
+static bool field_leaf(const pfmbem* h, int npts, FieldLeaf& fl) {
+  const Level& L = h->lev[h->D];
+  if (npts < 32 || h->hmax > 0.25 * L.d) return false;
+  fl.R = (h->tree == 1 ? 0.5 : 0.5 * sqrt(2.0)) * L.d;
+  const double kd = 2.0 * h->k * fl.R;
+  if (kd < 1e-6 || L.p < 20 || L.p < kd + 1.8 * pow(10.0, 2.0 / 3.0) * cbrt(kd)) return false;
+  const double far = (fl.R + 0.5 * h->hmax) / fmin(0.26, pow(10.0, -14.7 / (L.p + 1)));
+  fl.far2 = far * far;
+  fl.nleaf = L.nne;
+  fl.D = h->D;
+  fl.p = L.p;
+  fl.d = L.d;
+  fl.ne = L.ne;
+  fl.bb = L.box_begin;
+  fl.be = L.box_end;
+  fl.ctr = L.ctr;
+  double t = 1.0;
+  for (fl.nmin = 0; fl.nmin < L.p && t > 1e-16; ++fl.nmin) t *= 0.25 * kd / (fl.nmin + 1);
+  return true;
+}
+
+// Multipoles of the leaves by the rules 2, 3 and 4, and the leaves' element lengths.
+static void field_rules(pfmbem* h, FieldLeaf& fl, cplx* M, double2* hr) {
+  const Level& L = h->lev[h->D];
+  leaf_lengths_kernel<<<(fl.nleaf + 127) / 128, 128, 0, h->stream>>>(fl.nleaf, fl.ne, fl.bb, fl.be, h->s_h, hr);
+  for (int g = 2; g <= 4; ++g)
+    p2m_f64_kernel<<<fl.nleaf, 128, 0, h->stream>>>(fl.ne, fl.bb, fl.be, h->D, L.d, L.p, nullptr, g, h->k, h->eta,
+                                                    h->x0, h->y0, h->s_c, h->s_t, h->s_nu, h->s_h, h->dens,
+                                                    M + (size_t)(g - 2) * fl.nleaf * L.P, L.ctr);
+  fl.M = M;
+  fl.hr = hr;
 }
 
 // The tree's levels for the derivative at theta_l, or false where the direct sum is
@@ -3049,11 +3239,17 @@ cudaError_t k_field(pfmbem* h, int npts, const double2* pts, cplx* u, cplx* dudx
   const cplx* L0 = wide ? h->wide_ML + 2 * h->wide_ps + 1 : r.L;
   FieldTree ft;
   const bool tree = by_tree && !u && field_tree(h, ft);
-  // slices of a point's sum: about 32 warps per SM in all, at least 8 terms a lane
-  const int64_t terms = (int64_t)(2 * mdir + 1) * h->E;
-  const int nsl = tree ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>((152 * 32 + npts - 1) / npts, terms / 256));
+  FieldLeaf fl;
+  const bool leaf = !tree && field_leaf(h, npts, fl);
+  // slices of a point's sum: about 32 warps per SM in all, at least 8 terms a lane; by
+  // leaves about eight blocks per SM, at least a pair a thread
+  const int64_t terms = (int64_t)(2 * mdir + 1) * (leaf ? fl.nleaf : h->E);
+  const int nsl = tree ? 1
+                       : (int)std::max<int64_t>(1, leaf ? std::min<int64_t>((152 * 8 + npts - 1) / npts, terms / FL_NT)
+                                                        : std::min<int64_t>((152 * 32 + npts - 1) / npts, terms / 256));
   void* buf = nullptr;
-  cudaError_t e = cudaMallocAsync(&buf, sizeof(cplx) * 2 * (size_t)npts * (nsl + 1), h->stream);
+  const size_t npart = 2 * (size_t)npts * (nsl + 1), nrule = leaf ? 3 * (size_t)fl.nleaf * (2 * fl.p + 1) : 0;
+  cudaError_t e = cudaMallocAsync(&buf, sizeof(cplx) * (npart + nrule + (leaf ? fl.nleaf : 0)), h->stream);
   if (e != cudaSuccess) return e;
   cplx* part = static_cast<cplx*>(buf);
   prof_begin(h, PH_OUT);
@@ -3061,6 +3257,16 @@ cudaError_t k_field(pfmbem* h, int npts, const double2* pts, cplx* u, cplx* dudx
     field_tree_kernel<<<npts + (npts + FT_NT - 1) / FT_NT, FT_NT, 0, h->stream>>>(
         ft, npts, pts, h->k, h->eta, h->H, ox, oy, h->x0, h->y0, mdir, h->alpha, h->s_c, h->s_t, h->s_nu, h->s_h,
         h->dens, p0, w0, L0, part);
+  } else if (leaf) {
+    field_rules(h, fl, part + npart, reinterpret_cast<double2*>(part + npart + nrule));
+    auto launch = [&](auto kern) {
+      kern<<<npts * nsl + (npts + FL_NT - 1) / FL_NT, FL_NT, 0, h->stream>>>(
+          fl, npts, pts, nsl, h->k, h->eta, h->H, ox, oy, h->x0, h->y0, mdir, h->alpha, h->s_c, h->s_t, h->s_nu,
+          h->s_h, h->dens, p0, w0, L0, part);
+    };
+    if (u && dudx1) launch(field_leaf_kernel<true, true>);
+    else if (u) launch(field_leaf_kernel<true, false>);
+    else launch(field_leaf_kernel<false, true>);
   } else {
     const unsigned grid = (unsigned)(((int64_t)npts * nsl + 3) / 4 + (npts + 127) / 128);
     auto launch = [&](auto kern) {
