@@ -88,7 +88,8 @@ typedef struct {
                        At most the FP64 order; the FP64 refinement of a mixed solve
                        keeps the solution at the FP64 product's accuracy */
   int batch_group;  /* blocks per instance group of pfmbem_solve_batch's persistent launch;
-                       0 = 8 (raised to fit the coefficients of the tree's top level, one
+                       0 = 8, or equal shares of the chip for fewer instances than such
+                       groups (raised to fit the coefficients of the tree's top level, one
                        warp each).  A batch uses the largest value among its handles */
   int tree;         /* 0 = square quadtree over the block (default); 1 = regular-triangle
                        quadtree for hexagon lattices (Sec. 3.1, Fig. 5): every fiber in the

@@ -2036,9 +2036,6 @@ static pfmbem_status gmres(pfmbem* h, const cplx* b, cplx* x, double tol, int ma
 }
 
 // ============================================================== batched solve
-// Blocks per instance group of the persistent batched launch.
-constexpr int kBatchGroup = 8;
-
 // Lockstep iterative refinement over many handles: every instance is a small
 // state machine (outer FP64 residual, then Arnoldi steps of an inner GMRES on
 // the handle's operator precision); each lockstep phase enqueues one unit of
@@ -2226,7 +2223,6 @@ pfmbem_status pfmbem_solve_batch(int ninst, const pfmbem_t* hs, double* const* p
     static const char* gsenv = std::getenv("PFMBEM_BATCH_GROUP");
     int GS = 0;
     for (int i = 0; i < ninst; ++i) GS = std::max(GS, hs[i]->opt.batch_group);
-    if (GS <= 0) GS = kBatchGroup;
     if (gsenv) GS = std::max(1, std::atoi(gsenv));
     // longest first (LPT): the instances by element count, descending
     std::vector<int> order(ninst);
