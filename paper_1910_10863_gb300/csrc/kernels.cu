@@ -1810,7 +1810,8 @@ __global__ void to_f32_kernel(size_t n, const cplx* __restrict__ a, cplxf* __res
 __global__ void l2p_coef_kernel(int E, const int* __restrict__ sleaf, int D, double d, int p,
                                 const double* __restrict__ iwgt, double k, double x0, double y0,
                                 const double2* __restrict__ sc, const double2* __restrict__ snu,
-                                cplx* __restrict__ out, cplxf* __restrict__ outf, const double2* __restrict__ ctr) {
+                                cplx* __restrict__ out, cplxf* __restrict__ outf, const double2* __restrict__ ctr,
+                                size_t es, size_t cs) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= E) return;
   const int P = 2 * p + 1;
@@ -1834,12 +1835,12 @@ __global__ void l2p_coef_kernel(int E, const int* __restrict__ sleaf, int D, dou
     zp = zp * z;
   }
   const cplx nuc{nu.x, nu.y};
-  // coefficient-major: entry (q, l) of element s at (q P + l) E + s
+  // entry (q, l) of element s at s es + (q P + l) cs
   for (int l = -p; l <= p; ++l) {
     const double iw = iwgt[l + p];
     const cplx v = mul_i((0.25 * iw) * Jp[p + 1 + l]);
     const cplx dv = mul_i((0.125 * k * iw) * (nuc * Jp[p + l] - conj(nuc) * Jp[p + l + 2]));
-    const size_t i0 = (size_t)(l + p) * E + s, i1 = (size_t)(P + l + p) * E + s;
+    const size_t i0 = s * es + (l + p) * cs, i1 = s * es + (P + l + p) * cs;
     out[i0] = v;
     out[i1] = dv;
     if (outf) {
@@ -2300,7 +2301,7 @@ cudaError_t k_build_fmm_caches(pfmbem* h) {
   prof_begin(h, PH_SETUP);
   l2p_coef_kernel<<<(h->E + 127) / 128, 128, 0, h->stream>>>(h->E, h->s_leaf, h->D, leaf.d, leaf.p, leaf.iw_dev, h->k,
                                                              h->x0, h->y0, h->s_c, h->s_nu, h->l2p_c, h->l2p_cf,
-                                                             nullptr);
+                                                             nullptr, 1, h->E);
   if (h->l2p_cl)
     to_f32_kernel<<<std::min<size_t>((nc + 255) / 256, 4096), 256, 0, h->stream>>>(nc, h->l2p_c, h->l2p_cf,
                                                                                    h->l2p_cl);
@@ -2521,7 +2522,7 @@ cudaError_t k_tri_caches(pfmbem* h) {
       h->E, h->s_leaf, h->D, leaf.d, leaf.p, leaf.iw_dev, h->g_far, h->k, h->eta, h->x0, h->y0, h->s_c, h->s_t,
       h->s_nu, h->s_h, h->p2m_c, leaf.ctr);
   l2p_coef_kernel<<<(h->E + 127) / 128, 128, 0, st>>>(h->E, h->s_leaf, h->D, leaf.d, leaf.p, leaf.iw_dev, h->k, h->x0,
-                                                      h->y0, h->s_c, h->s_nu, h->l2p_c, nullptr, leaf.ctr);
+                                                      h->y0, h->s_c, h->s_nu, h->l2p_c, nullptr, leaf.ctr, 2 * leaf.P, 1);
   prof_end(h, PH_SETUP);
   e = k_build_caches(h, nullptr);
   if (e != cudaSuccess) return e;

@@ -3479,11 +3479,10 @@ __global__ void __launch_bounds__(1024) tri_l2l_dd_kernel(const int* __restrict_
   }
 }
 
-// Threads over the coefficients by shares of a column: short chains on levels of few
-// boxes (below eight blocks of 256 threads per SM), a block of four shares elsewhere.
-static dim3 tri_block(int P, int nbox) {
+// Threads over the coefficients by shares of a column, within the block's limit.
+static dim3 tri_block(int P, int shares) {
   const int x = ((P + 31) / 32) * 32;
-  return dim3(x, std::max(1, std::min(nbox < 8 * 152 ? TRI_Y : 4, 1024 / x)));
+  return dim3(x, std::max(1, std::min(shares, 1024 / x)));
 }
 
 // ------------------------------------- triangle tree: tables as double-float words
@@ -3574,40 +3573,37 @@ __global__ void __launch_bounds__(256) tri_fiber_kernel(const int* __restrict__ 
 
 // L2P and the near sums (U, already there), added to y in the caller's order:
 // y_e += alpha^{m0} (U + U', c2 (dU + dU')), U'_s = sum_l c[s][0][l] L_l, dU'_s =
-// sum_l c[s][1][l] L_l with the words of c.  One block per leaf, 16 elements by 16
-// shares of the coefficients: the words lie element by element (entry (q, l) of
-// element s at (q P + l) E + s), so the elements of a leaf are read together.
-__global__ void __launch_bounds__(256) tri_l2p_add_kernel(
-    const int* __restrict__ ne, const int* __restrict__ bb, const int* __restrict__ be, int P, int E,
-    const float4* __restrict__ coef, const cplx* __restrict__ L, const cplx* __restrict__ U,
-    const int* __restrict__ perm, const cplx* __restrict__ sph, cplx c2, cplx* __restrict__ y) {
-  __shared__ float4 sL[PF_NCOEF], red[2][16][17];
-  const int box = ne[blockIdx.x], el = threadIdx.x & 15, sl = threadIdx.x >> 4;
-  for (int l = threadIdx.x; l < P; l += 256) sL[l] = dd_word(L[(size_t)box * P + l]);
-  for (int s0 = bb[box]; s0 < be[box]; s0 += 16) {
-    const int s = s0 + el;
-    __syncthreads();
+// sum_l c[s][1][l] L_l with the words of c, an element's 2 P words together.  A warp
+// per element; one warp of the block does the FP64 ends of its eight elements (a warp
+// instruction of the FP64 pipe costs the same for one lane as for sixteen).  With the
+// coefficients element by element (16 bytes of each line for a leaf of one) 16384
+// elements took 78 to 134 us.
+__global__ void __launch_bounds__(256) tri_l2p_add_kernel(int E, const int* __restrict__ sleaf, int P,
+                                                          const float4* __restrict__ coef,
+                                                          const cplx* __restrict__ L, const cplx* __restrict__ U,
+                                                          const int* __restrict__ perm, const cplx* __restrict__ sph,
+                                                          cplx c2, cplx* __restrict__ y) {
+  __shared__ double so[8][4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, s = blockIdx.x * 8 + warp;
+  if (s < E) {
+    const cplx* Lb = L + (size_t)sleaf[s] * P;
+    const float4* cs = coef + (size_t)s * 2 * P;
     dflt a{0, 0}, b{0, 0}, c{0, 0}, d{0, 0};
-    if (s < be[box])
-#pragma unroll 4
-      for (int l = sl; l < P; l += 16) {
-        const float4 v = sL[l];
-        dd_cmac(a, b, coef[(size_t)l * E + s], v);
-        dd_cmac(c, d, coef[(size_t)(P + l) * E + s], v);
-      }
-    red[0][sl][el] = make_float4(a.h, b.h, a.l, b.l);
-    red[1][sl][el] = make_float4(c.h, d.h, c.l, d.l);
-    __syncthreads();
-    if (sl < 2 && s < be[box]) {
-      dflt u{0, 0}, v{0, 0};
-      for (int q = 0; q < 16; ++q) {
-        const float4 w = red[sl][q][el];
-        u = dd_add(u, dflt{w.x, w.z});
-        v = dd_add(v, dflt{w.y, w.w});
-      }
-      const cplx t = conj(sph[s]) * (U[2 * s + sl] + cplx{dd_value(u), dd_value(v)});   // |sph| = 1
-      y[2 * perm[s] + sl] += sl ? c2 * t : t;
+#pragma unroll 2
+    for (int l = lane; l < P; l += 32) {
+      const float4 u = cs[l], w = cs[P + l], v = dd_word(Lb[l]);
+      dd_cmac(a, b, u, v);
+      dd_cmac(c, d, w, v);
     }
+    const dflt r = dd_wsum4(a, b, c, d, lane);
+    if ((lane & 7) == 0) so[warp][lane >> 3] = dd_value(r);
+  }
+  __syncthreads();
+  const int t = blockIdx.x * 8 + (threadIdx.x >> 1), q = threadIdx.x & 1;
+  if (threadIdx.x < 16 && t < E) {
+    const double* v = so[threadIdx.x >> 1] + 2 * q;
+    const cplx w = conj(sph[t]) * (U[2 * t + q] + cplx{v[0], v[1]});   // |sph| = 1
+    y[2 * perm[t] + q] += q ? c2 * w : w;
   }
 }
 
@@ -3640,17 +3636,20 @@ cudaError_t k_tri_fiber(pfmbem* h, const cplx* x, cplx* y, cudaStream_t st) {
 
 cudaError_t k_tri_l2p(pfmbem* h, cplx* y) {
   const Level& leaf = h->lev[h->D];
-  tri_l2p_add_kernel<<<leaf.nne, 256, 0, h->stream>>>(leaf.ne, leaf.box_begin, leaf.box_end, leaf.P, h->E,
-                                                      reinterpret_cast<const float4*>(h->l2p_c), leaf.L, h->U,
-                                                      h->s_perm, h->s_ph, cplx{h->c2re, h->c2im}, y);
+  tri_l2p_add_kernel<<<(h->E + 7) / 8, 256, 0, h->stream>>>(h->E, h->s_leaf, leaf.P,
+                                                            reinterpret_cast<const float4*>(h->l2p_c), leaf.L, h->U,
+                                                            h->s_perm, h->s_ph, cplx{h->c2re, h->c2im}, y);
   return cudaGetLastError();
 }
 
 cudaError_t k_tri_m2m_dd(pfmbem* h, int l) {
   const Level& a = h->lev[l];
   const Level& c = h->lev[l + 1];
+  // 16 shares where the boxes are few (the chain over a box's children is the level's
+  // time: 64 to 500 boxes 18 to 28 us, by 4 shares 32 us); 1139 boxes take 51 us by 16
+  // and 34 us by 4, for the shares' ends then fill the chip
   const int nch = l == 0 ? 6 : 4;
-  const dim3 nt = tri_block(a.P, a.nne);
+  const dim3 nt = tri_block(a.P, a.nne <= 4 * 152 ? TRI_Y : 4);
   const size_t smem = sizeof(float4) * std::max((size_t)nch * c.P, (size_t)nt.y * a.P);
   tri_m2m_dd_kernel<<<a.nne, nt, smem, h->stream>>>(a.ne, a.P, c.P, a.tri_nop, a.tri_m2m_hl, c.box_begin, c.box_end,
                                                     c.M, a.M, nch, c.pidx, a.L);
@@ -3660,7 +3659,7 @@ cudaError_t k_tri_m2m_dd(pfmbem* h, int l) {
 cudaError_t k_tri_l2l_dd(pfmbem* h, int l) {
   const Level& a = h->lev[l];
   const Level& pa = h->lev[l - 1];
-  const dim3 nt = tri_block(a.P, a.nne);
+  const dim3 nt = tri_block(a.P, 4);
   const size_t smem = sizeof(float4) * ((size_t)pa.P + (size_t)nt.y * a.P);
   tri_l2l_dd_kernel<<<a.nne, nt, smem, h->stream>>>(a.ne, a.P, pa.P, pa.tri_nop, pa.tri_l2l_hl, pa.L, a.L,
                                                     l == 1 ? 6 : 4, a.pidx);
