@@ -1434,41 +1434,86 @@ __global__ void near_build_kernel(const int* __restrict__ ne, const int* __restr
 }
 
 // The near-field pairs that no table covers, one thread each: the element
-// integrals by the Gauss ladder (as above), written into their blocks.
-__global__ void near_direct_kernel(const unsigned long long* __restrict__ queue, const unsigned* __restrict__ qlen,
-                                   unsigned qcap, const int* __restrict__ ne, const int* __restrict__ bb,
-                                   const int64_t* __restrict__ base, const int* __restrict__ sbase,
-                                   const int* __restrict__ srcf, const int* __restrict__ srcm, double k, double eta,
-                                   double H, cplx alpha, const double2* __restrict__ sc,
-                                   const double2* __restrict__ st, const double2* __restrict__ snu,
-                                   const double* __restrict__ sh, cplx* __restrict__ val, cplxf* __restrict__ valf,
-                                   cplxf* __restrict__ vall, unsigned long long* __restrict__ stat) {
+// integrals by the Gauss ladder (as above), written into their blocks.  A block sorts
+// its batch by the rule, the largest first, so that the threads of a warp take equally
+// many nodes: the FP64 pipe bounds it, and in the queue's order a warp took as long as
+// its nearest pair.
+constexpr int ND_NT = 128, ND_MAX = 1024;
+__global__ void __launch_bounds__(ND_NT) near_direct_kernel(
+    const unsigned long long* __restrict__ queue, const unsigned* __restrict__ qlen, unsigned qcap,
+    const int* __restrict__ ne, const int* __restrict__ bb, const int64_t* __restrict__ base,
+    const int* __restrict__ sbase, const int* __restrict__ srcf, const int* __restrict__ srcm, double k, double eta,
+    double H, cplx alpha, const double2* __restrict__ sc, const double2* __restrict__ st,
+    const double2* __restrict__ snu, const double* __restrict__ sh, cplx* __restrict__ val, cplxf* __restrict__ valf,
+    cplxf* __restrict__ vall, unsigned long long* __restrict__ stat) {
+  __shared__ unsigned long long s_w[ND_MAX];
+  __shared__ unsigned char s_g[ND_MAX];
+  __shared__ int s_cnt[PF_GLMAX + 1], s_off[PF_GLMAX + 1];
   const unsigned n = min(*qlen, qcap);
+  // pairs of a batch: the block's share, in whole passes of the block
+  const unsigned share = (n + gridDim.x - 1) / gridDim.x;
+  const int batch = (int)min((unsigned)ND_MAX, max(1u, (share + ND_NT - 1) / ND_NT) * ND_NT);
   unsigned long long npair = 0, nquad = 0;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const unsigned long long w = queue[i];
-    const int li = (int)(w >> 40), t = (int)((w >> 24) & 0xFFFF), j = (int)(w & 0xFFFFFF);
-    const int s = bb[ne[li]] + t;
-    const int j0 = sbase[li], ns = sbase[li + 1] - j0;
-    const int f = srcf[j0 + j], m = srcm[j0 + j];
-    const double2 x = sc[s], nx = snu[s];
-    double2 c = sc[f];
-    c.y += m * H;
-    const double hh = sh[f];
-    const double q = sqrt((x.x - c.x) * (x.x - c.x) + (x.y - c.y) * (x.y - c.y)) / hh;
-    const int g = gl_order(q, 0);
-    ++npair;
-    nquad += g;
-    cplx S{0, 0}, Dv{0, 0}, K{0, 0}, T{0, 0};
-    pair4_f64(k, x, nx, c, st[f], snu[f], hh, g, S, Dv, K, T);
-    const cplx ph = mul_i(0.25 * ipow_phase(alpha, m));      // (i/4) alpha^m
-    const cplx b[4] = {ph * Dv, (-eta) * mul_i(ph * S), ph * T, (-eta) * mul_i(ph * K)};
-    const int64_t o = base[li] + ((int64_t)t * ns + j) * 4;
-    for (int q2 = 0; q2 < 4; ++q2) {
-      if (val) val[o + q2] = b[q2];
-      if (valf) valf[o + q2] = cplxf{(float)b[q2].re, (float)b[q2].im};
-      vall[o + q2] = split_lo(b[q2]);
+  for (int64_t b0 = (int64_t)blockIdx.x * batch; b0 < n; b0 += (int64_t)gridDim.x * batch) {
+    const int m0 = (int)min((int64_t)batch, n - b0);
+    if (threadIdx.x <= PF_GLMAX) s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned long long wr[ND_MAX / ND_NT];
+    int key[ND_MAX / ND_NT];           // rule and place among its like
+#pragma unroll
+    for (int r = 0; r < ND_MAX / ND_NT; ++r) {
+      const int e = r * ND_NT + (int)threadIdx.x;
+      if (e >= m0) continue;
+      const unsigned long long w = queue[b0 + e];
+      const int li = (int)(w >> 40), t = (int)((w >> 24) & 0xFFFF), j = (int)(w & 0xFFFFFF);
+      const int f = srcf[sbase[li] + j];
+      const double2 x = sc[bb[ne[li]] + t];
+      double2 c = sc[f];
+      c.y += srcm[sbase[li] + j] * H;
+      const int g = gl_order(sqrt((x.x - c.x) * (x.x - c.x) + (x.y - c.y) * (x.y - c.y)) / sh[f], 0);
+      wr[r] = w;
+      key[r] = (g << 16) | atomicAdd(&s_cnt[g], 1);
     }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int g = PF_GLMAX, o = 0; g >= 0; --g) {
+        s_off[g] = o;
+        o += s_cnt[g];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ND_MAX / ND_NT; ++r)
+      if (r * ND_NT + (int)threadIdx.x < m0) {
+        const int g = key[r] >> 16, o = s_off[g] + (key[r] & 0xFFFF);
+        s_w[o] = wr[r];
+        s_g[o] = (unsigned char)g;
+      }
+    __syncthreads();
+    for (int e = threadIdx.x; e < m0; e += ND_NT) {
+      const unsigned long long w = s_w[e];
+      const int li = (int)(w >> 40), t = (int)((w >> 24) & 0xFFFF), j = (int)(w & 0xFFFFFF);
+      const int s = bb[ne[li]] + t;
+      const int j0 = sbase[li], ns = sbase[li + 1] - j0;
+      const int f = srcf[j0 + j], m = srcm[j0 + j];
+      const double2 x = sc[s], nx = snu[s];
+      double2 c = sc[f];
+      c.y += m * H;
+      const double hh = sh[f];
+      const int g = s_g[e];
+      ++npair;
+      nquad += g;
+      cplx S{0, 0}, Dv{0, 0}, K{0, 0}, T{0, 0};
+      pair4_f64(k, x, nx, c, st[f], snu[f], hh, g, S, Dv, K, T);
+      const cplx ph = mul_i(0.25 * ipow_phase(alpha, m));      // (i/4) alpha^m
+      const cplx b[4] = {ph * Dv, (-eta) * mul_i(ph * S), ph * T, (-eta) * mul_i(ph * K)};
+      const int64_t o = base[li] + ((int64_t)t * ns + j) * 4;
+      for (int q2 = 0; q2 < 4; ++q2) {
+        if (val) val[o + q2] = b[q2];
+        if (valf) valf[o + q2] = cplxf{(float)b[q2].re, (float)b[q2].im};
+        vall[o + q2] = split_lo(b[q2]);
+      }
+    }
+    __syncthreads();
   }
   if (stat) {
     npair = warp_sum_u64(npair);
@@ -1724,7 +1769,7 @@ cudaError_t k_build_caches(pfmbem* h, cudaEvent_t ktab_done) {
   prof_end(h, PH_BUILD);
   trace(h, st, "near: near_build done");
   prof_begin(h, PH_BUILD);
-  near_direct_kernel<<<1216, 128, 0, st>>>(h->nq, h->nq_len, h->nq_cap, leaf.ne, leaf.box_begin, h->nc_base,
+  near_direct_kernel<<<1216, ND_NT, 0, st>>>(h->nq, h->nq_len, h->nq_cap, leaf.ne, leaf.box_begin, h->nc_base,
                                            h->nc_sbase, h->nc_src, h->nc_img, h->k, h->eta, h->H, h->alpha, h->s_c,
                                            h->s_t, h->s_nu, h->s_h, h->nc_val, h->nc_valf, h->nc_vall,
                                            h->stat_dev);
