@@ -410,6 +410,7 @@ void ensure_gauss() {
   gl_thresholds(1e-14, g_thr64);
   gl_thresholds(3e-8, g_thr32);
   k_upload_gauss(x.data(), w.data(), g_thr64, g_thr32);
+  k_upload_series();
   g_gauss_ready_dev = dev;
 }
 

@@ -414,6 +414,7 @@ cudaError_t k_coefficients(pfmbem* h, const cplx* psi, int norders, const int* o
 
 // ------------------------------------------------------------ kernel launches
 void k_upload_gauss(const double* x, const double* w, const double* thr64, const double* thr32);
+void k_upload_series();
 cudaError_t k_self_terms(pfmbem* h);
 // translation tables of all levels (kernels.cu)
 struct TableLevels {

@@ -860,11 +860,67 @@ __device__ __forceinline__ void bessel01(double x, double& J0, double& J1, doubl
   Y1 = Q1 * d - P1 * c;
 }
 
+// The same four by the ascending series with psi(m+1) = H_m - gamma to x = 4 and CUDA's
+// functions above, for the scattered field itself: where a density radiates almost
+// nothing u cancels to 1e-8 of its terms, and another rounding of these functions shows
+// at 1e-8 of u (the joint interpolants take half the time).  Per-term constants of the
+// series, m = 1..39: 1/m^2, 1/(m(m+1)), H_m and 2 H_m + 1/(m+1) - 2 gamma.
+__constant__ double c_ser_im2[40], c_ser_imm1[40], c_ser_H[40], c_ser_y1[40];
+
+void k_upload_series() {
+  double im2[40] = {0}, imm1[40] = {0}, H[40] = {0}, y1c[40] = {0};
+  const double EG = 0.57721566490153286061;
+  double Hm = 0.0;
+  for (int m = 1; m < 40; ++m) {
+    im2[m] = 1.0 / ((double)m * m);
+    imm1[m] = 1.0 / ((double)m * (m + 1));
+    Hm += 1.0 / m;
+    H[m] = Hm;
+    y1c[m] = 2.0 * Hm + 1.0 / (m + 1) - 2.0 * EG;
+  }
+  cudaMemcpyToSymbol(c_ser_im2, im2, sizeof(im2));
+  cudaMemcpyToSymbol(c_ser_imm1, imm1, sizeof(imm1));
+  cudaMemcpyToSymbol(c_ser_H, H, sizeof(H));
+  cudaMemcpyToSymbol(c_ser_y1, y1c, sizeof(y1c));
+}
+
+__device__ __forceinline__ void bessel01_series(double x, double& J0, double& J1, double& Y0, double& Y1) {
+  if (x > 4.0) {
+    J0 = j0(x); J1 = j1(x); Y0 = y0(x); Y1 = y1(x);
+    return;
+  }
+  const double h = 0.5 * x, h2 = h * h;
+  const double EG = 0.57721566490153286061;
+  // a_m = (-1)^m (x/2)^{2m} / (m!)^2,  b_m = (-1)^m (x/2)^{2m} / (m! (m+1)!)
+  double a = 1.0, b = 1.0;
+  double sJ0 = 1.0, sJ1 = 1.0, sY0 = 0.0, sY1 = -(2.0 * (-EG) + 1.0);  // m = 0 terms
+  // Y1 series term: (psi(m+1) + psi(m+2)) b_m with psi(m+1) = H_m - gamma
+  // the number of terms for |term| < 1e-17 grows with x; bound it from x
+  const int mmax = x < 0.5 ? 10 : (x < 1.5 ? 15 : (x < 3.0 ? 21 : 27));
+#pragma unroll 1
+  for (int m = 1; m < mmax; ++m) {
+    a *= -h2 * c_ser_im2[m];
+    b *= -h2 * c_ser_imm1[m];
+    sJ0 += a;
+    sJ1 += b;
+    sY0 = fma(-c_ser_H[m], a, sY0);           // (-1)^{m+1} H_m (x/2)^{2m}/(m!)^2
+    sY1 = fma(-c_ser_y1[m], b, sY1);
+  }
+  const double L = log(h);
+  J0 = sJ0;
+  J1 = h * sJ1;
+  Y0 = (2.0 / M_PI) * ((L + EG) * J0 + sY0);
+  // Y1 = -2/(pi x) + (2/pi) ln(x/2) J1 - (1/pi) sum (psi(m+1) + psi(m+2)) b_m (x/2)
+  Y1 = -2.0 / (M_PI * x) + (2.0 / M_PI) * L * J1 + (1.0 / M_PI) * h * sY1;
+}
+
 // ---------------------------------------------------------------- pair integrals
 // Element integrals of (i/4)H0(kap|x-y|) (S), its d/dnu_y (D), d/dnu_x (K) and
 // d2/dnu_x dnu_y (T) over the flat element c + s t, |s| <= h/2, by g-point
 // Gauss-Legendre; the factor i/4 is applied by the caller.  Nodes q0, q0 + qs,
-// ... only (a share of the rule, for callers that split it over lanes).
+// ... only (a share of the rule, for callers that split it over lanes); SER: the Bessel
+// functions by bessel01_series.
+template <bool SER = false>
 __device__ __forceinline__ void pair4_f64(double kap, double2 x, double2 nx, double2 c, double2 t, double2 ny,
                                           double h, int g, cplx& S, cplx& D, cplx& K, cplx& T, int q0 = 0,
                                           int qs = 1) {
@@ -879,7 +935,8 @@ __device__ __forceinline__ void pair4_f64(double kap, double2 x, double2 nx, dou
     double ir = 1.0 / r;
     double kr = kap * r;
     double J0, J1, Y0, Y1;
-    bessel01(kr, J0, J1, Y0, Y1);
+    if (SER) bessel01_series(kr, J0, J1, Y0, Y1);
+    else bessel01(kr, J0, J1, Y0, Y1);
     double zy = (z1 * ny.x + z2 * ny.y) * ir;
     double zx = (z1 * nx.x + z2 * nx.y) * ir;
     S += wq * cplx{J0, Y0};
@@ -966,11 +1023,12 @@ __global__ void p2m_f64_kernel(const int* __restrict__ ne, const int* __restrict
     cplx a = (cw * 0.5 * k) * ph;
     cplx bcoef = (-eta * cw) * mul_i(va);
     cplx nuc{nu.x, nu.y};
-    for (int n = -p; n <= p; ++n) {
-      cplx v = a * (conj(nuc) * Jm[p + n] - nuc * Jm[p + n + 2]) + bcoef * Jm[p + n + 1];
-      double iw = wgt ? 1.0 / wgt[n + p] : 1.0;
-      atomicAdd(&acc[2 * (n + p)], v.re * iw);
-      atomicAdd(&acc[2 * (n + p) + 1], v.im * iw);
+    // every thread begins at another coefficient: in step they would all add to one word
+    for (int i = 0, j = threadIdx.x % P; i < P; ++i, j = j + 1 < P ? j + 1 : 0) {
+      cplx v = a * (conj(nuc) * Jm[j] - nuc * Jm[j + 2]) + bcoef * Jm[j + 1];
+      double iw = wgt ? 1.0 / wgt[j] : 1.0;
+      atomicAdd(&acc[2 * j], v.re * iw);
+      atomicAdd(&acc[2 * j + 1], v.im * iw);
     }
   }
   __syncthreads();
@@ -1538,23 +1596,27 @@ __global__ void __launch_bounds__(ND_NT) near_direct_kernel(
 // dl = f - f0 (zero for dl = 0).  Rotating the fiber by one element maps it onto
 // itself, so element pair (e, e + dl) has the integrals of (f0, f0 + dl) and the
 // near-field build reads same-fiber pairs from this table.
-// FB_SPLIT consecutive lanes share one (row element e, source f) pair and take
-// every FB_SPLIT-th Gauss node; the partial sums meet by shuffles.
+// SP consecutive lanes share one (row element e, source f) pair and take every SP-th
+// Gauss node; the partial sums meet by shuffles.  Four where the rows are few (regular
+// polygons keep one: a pair's chain of nodes is then the time), one elsewhere: the FP64
+// pipe bounds it, a rule of three nodes left a lane of four idle, and the end of a pair
+// (the sums' shuffles and the products by c2) costs a warp the same for 8 pairs as for 32.
 // A regular polygon is also symmetric under the reflection through the
 // midpoint of its first element and the centre: it maps source f0 + dl onto
 // f0 + N - dl and keeps both normals outward, and the Gauss rule is symmetric,
 // so the first element's row (both planes) takes the integrals of dl <= N/2
 // and writes each also at N - dl.
-constexpr int FB_SPLIT = 4;
 
+template <int SP>
 __device__ __forceinline__ void group_sum(cplx& v) {
 #pragma unroll
-  for (int o = 1; o < FB_SPLIT; o <<= 1) {
+  for (int o = 1; o < SP; o <<= 1) {
     v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
     v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
   }
 }
 
+template <int SP>
 __global__ void fiber_build_kernel(const int* __restrict__ rows, const int* __restrict__ fib,
                                    const int* __restrict__ foff, const int64_t* __restrict__ fbase, double k,
                                    double k1, double eta, double rho, cplx c2, const double2* __restrict__ oc,
@@ -1570,9 +1632,9 @@ __global__ void fiber_build_kernel(const int* __restrict__ rows, const int* __re
   const int64_t kb = kbase[fb];
   if (ktab && kb < 0) return;                      // uniform over the block
   const bool mir = kb >= 0 && el == 0;             // mirrored half row (regular polygon)
-  if (mir && (int)blockIdx.y * (int)(blockDim.x / FB_SPLIT) > N / 2) return;   // uniform over the block
-  const int part = threadIdx.x % FB_SPLIT;
-  const int fl = blockIdx.y * (blockDim.x / FB_SPLIT) + threadIdx.x / FB_SPLIT;
+  if (mir && (int)blockIdx.y * (int)(blockDim.x / SP) > N / 2) return;   // uniform over the block
+  const int part = threadIdx.x % SP;
+  const int fl = blockIdx.y * (blockDim.x / SP) + threadIdx.x / SP;
   const bool lead = part == 0;
   unsigned long long np = 0, nq = 0;
   const bool on = fl < N && !(mir && fl > N / 2);
@@ -1590,12 +1652,12 @@ __global__ void fiber_build_kernel(const int* __restrict__ rows, const int* __re
       np = fm >= 0 ? 2 : 1;
       nq = fm >= 0 ? 2 * g : g;
     }
-    pair4_f64(ktab ? k : k1, xe, nxe, c, tf, nf, hh, g, S, Dv, K, T, part, FB_SPLIT);
+    pair4_f64(ktab ? k : k1, xe, nxe, c, tf, nf, hh, g, S, Dv, K, T, part, SP);
   }
-  group_sum(S);
-  group_sum(Dv);
-  group_sum(K);
-  group_sum(T);
+  group_sum<SP>(S);
+  group_sum<SP>(Dv);
+  group_sum<SP>(K);
+  group_sum<SP>(T);
   if (on && lead) {
     if (ktab) {
       cplx* tv = kval + 4 * (kb + fl);
@@ -1713,7 +1775,9 @@ __global__ void near_sources_kernel(const int* __restrict__ nl_ptr, const int* _
 static void fiber_build_plane(pfmbem* h, bool ktab, cudaStream_t st) {
   cplx c2{h->c2re, h->c2im};
   prof_begin(h, PH_BUILD);
-  fiber_build_kernel<<<dim3(h->nfb_rows, (h->max_fiber + 128 / FB_SPLIT - 1) / (128 / FB_SPLIT), 1), 128, 0, st>>>(
+  const int sp = (int64_t)h->nfb_rows * h->max_fiber >= 152 * 2048 ? 1 : 4;   // pairs for every resident thread
+  auto kern = sp == 1 ? fiber_build_kernel<1> : fiber_build_kernel<4>;
+  kern<<<dim3(h->nfb_rows, (h->max_fiber + 128 / sp - 1) / (128 / sp), 1), 128, 0, st>>>(
       h->fb_rows, h->o_fiber, h->fib_off, h->fb_base, h->k, h->k1, h->eta, h->rho, c2, h->o_c, h->o_t, h->o_nu,
       h->o_h, h->self4, h->kt_base, h->kt_val, h->kt_sval, h->kt_svalf, h->kt_svall, h->fb_val, h->fb_valf,
       h->stat_dev, ktab ? 1 : 0);
@@ -2838,10 +2902,12 @@ __global__ void field_finish_kernel(int npts, const double2* __restrict__ pts, i
 // One warp per (point, slice): slice q of nsl takes every nsl-th group of 32 of
 // the (element, image) pairs and leaves its sums in part[point][q]; the local
 // expansions are separate threads (the last blocks) and go to part[point][nsl];
-// field_finish_kernel adds a point's parts in order.  Bound by the FP64 pipe; one
-// warp per point left most of the chip idle below some thousand points, and its
-// lane 0 alone evaluated the local expansion (1024 points on 16384 elements: 74 ->
-// 64 ms, 73 points on 9 k elements: 37 -> 22 ms with the joint Bessel functions).
+// field_finish_kernel adds a point's parts in order.  Bound by the FP64 pipe.  The
+// derivative alone takes slices, for one warp per point leaves most of the chip idle
+// below some thousand points.  u takes one slice and the series' Bessel functions: its
+// terms are of the size of 1 where it may be 1e-8, so that another order of the sum
+// shows at 2e-9 to 7e-9 of u (1024 points on 16384 elements: 117 ms; 74 ms with the
+// joint interpolants, 64 ms with slices too).
 template <bool WU, bool WD>
 __global__ void __launch_bounds__(128) field_direct_kernel(
     int npts, const double2* __restrict__ pts, int nsl, int E, double k, double eta, double H, double ox, double oy,
@@ -2869,7 +2935,7 @@ __global__ void __launch_bounds__(128) field_direct_kernel(
     const double q = sqrt((x.x - c.x) * (x.x - c.x) + (x.y - c.y) * (x.y - c.y)) / hh;
     const int g = gl_order(q, 0);
     cplx S{0, 0}, Dv{0, 0}, K{0, 0}, T{0, 0};
-    pair4_f64(k, x, nx, c, st[f], snu[f], hh, g, S, Dv, K, T);
+    pair4_f64<WU>(k, x, nx, c, st[f], snu[f], hh, g, S, Dv, K, T);
     const cplx ph = ipow_phase(alpha, m);
     if (WU) acc += ph * (Dv * dens[2 * f] - eta * mul_i(S * dens[2 * f + 1]));
     if (WD) dacc += ph * (T * dens[2 * f] - eta * mul_i(K * dens[2 * f + 1]));
@@ -2918,12 +2984,10 @@ struct FieldTree {
   const double2* ctr[PF_MAXLEVEL + 1]; // box centres (triangle tree), null: from the Morton code
 };
 
-// sum_{|n| <= q} c_n H^+_n(k v) (WU) and its x1-derivative (WD), c_n = w_n M_n, or M_n
-// without weights; q <= p, the order of M.
-template <bool WU, bool WD>
-__device__ __forceinline__ void multipole_eval(double k, double vx, double vy, int p, int q,
-                                               const double* __restrict__ w, const cplx* __restrict__ M, cplx& u,
-                                               cplx& d) {
+// x1-derivative of sum_{|n| <= q} c_n H^+_n(k v), c_n = w_n M_n, or M_n without weights;
+// q <= p, the order of M.
+__device__ __forceinline__ cplx multipole_dx1(double k, double vx, double vy, int p, int q,
+                                              const double* __restrict__ w, const cplx* __restrict__ M) {
   const double r2 = vx * vx + vy * vy, ir = rsqrt(r2), x = k * r2 * ir;
   const cplx z{vx * ir, vy * ir};
   double J0, J1, Y0, Y1;
@@ -2937,15 +3001,13 @@ __device__ __forceinline__ void multipole_eval(double k, double vx, double vy, i
   // coefficients around +-n: a_n = c_n, b_n = c_-n
   const cplx c0 = coef(0);
   cplx am = c0, a = coef(1), b = c0, bn = coef(-1);    // am = c_{n-1}, a = c_n, b = c_{-(n-1)}, bn = c_{-n}
-  if (WU) u = hm * c0;
-  if (WD) d = hm * (a - bn);                   // m = 0: c_1 - c_-1
+  cplx d = hm * (a - bn);                      // m = 0: c_1 - c_-1
   double sg = -1.0;
-  for (int n = 1; n <= q + (WD ? 1 : 0); ++n) {
+  for (int n = 1; n <= q + 1; ++n) {
     zp = zp * z;
     const cplx hp = h * zp, hn = sg * (h * conj(zp));   // H^+_n, H^+_-n
     const cplx a2 = coef(n + 1), b2 = coef(-n - 1);      // c_{n+1}, c_{-(n+1)}
-    if (WU) u += hp * a + hn * bn;
-    if (WD) d += hp * (a2 - am) + hn * (b - b2);
+    d += hp * (a2 - am) + hn * (b - b2);
     am = a;
     a = a2;
     b = bn;
@@ -2955,7 +3017,7 @@ __device__ __forceinline__ void multipole_eval(double k, double vx, double vy, i
     hm = h;
     h = hnext;
   }
-  if (WD) d = (0.5 * k) * d;
+  return (0.5 * k) * d;
 }
 
 __global__ void __launch_bounds__(FT_NT) field_tree_kernel(
@@ -2994,10 +3056,8 @@ __global__ void __launch_bounds__(FT_NT) field_tree_kernel(
       }
       const double vx = x.x - cx, vy = x.y - (cy + m * H);
       if (vx * vx + vy * vy >= ft.far2[l]) {
-        cplx u, du;
-        multipole_eval<false, true>(k, vx, vy, ft.p[l], ft.p[l], ft.w[l],
-                                    ft.M[l] + (size_t)box * (2 * ft.p[l] + 1), u, du);
-        dacc += ipow_phase(alpha, m) * du;
+        dacc += ipow_phase(alpha, m) *
+                multipole_dx1(k, vx, vy, ft.p[l], ft.p[l], ft.w[l], ft.M[l] + (size_t)box * (2 * ft.p[l] + 1));
       } else {
         const int o = atomicAdd(&s_n[cur], 1);
         if (o < FT_CAP) {
@@ -3049,21 +3109,21 @@ __global__ void __launch_bounds__(FT_NT) field_tree_kernel(
   }
 }
 
-// u and its x1-derivative through the multipoles of the leaves, of the same quadrature
-// as the direct sum.  Where a density radiates almost nothing u cancels to 1e-6 of its
-// terms and the Gauss ladder's remainders (1e-14 of an element's term) show, so a leaf
-// enters as a whole only where the ladder gives all its elements one rule g = 2, 3 or 4
-// (54 h <= r for g = 3, 790 h for 2; other leaves, and those nearer than the expansion
-// allows, go element by element), by the multipoles of that rule's nodes, taken once per
-// call (field_rules).  The expansion ends where its remainder is below 10^-15 of the
-// leaf's field: at order q with (R / r)^q and (k R / 2)^q / q! below it.
+// The x1-derivative at many points through the multipoles of the leaves, of the same
+// quadrature as the direct sum: a leaf enters as a whole where the ladder gives all its
+// elements one rule g = 2, 3 or 4 (54 h <= r for g = 3, 790 h for 2; other leaves, and
+// those nearer than the expansion allows, go element by element), by the multipoles of
+// that rule's nodes, taken once per call (field_rules).  The expansion ends at the order
+// q with (R / r)^q and (k R / 2)^q / q! below 10^-18: a dipole's remainder is q r / R
+// times that, 10^-16 of the leaf's field.  The field u stays directly summed: where a
+// density radiates almost nothing it cancels to 1e-8 of its terms, and any other rounding
+// of these shows at 3e-9 to 9e-9 of u (of the derivative at 1e-10).
 // A block takes slice sl of nsl of a point's (leaf, image) pairs; the pairs that go by
 // elements are collected in shared memory and summed together when the list fills.
 // Bound by the FP64 pipe: some 500 instructions a leaf, against 500 to 700 an element.
-// 1024 points on 16384 elements: 8.0 ms, 64 ms element by element.
 constexpr int FL_NT = 256, FL_CAP = 1024;
 struct FieldLeaf {
-  int nleaf, D, p, nmin;                 // nmin: order from which (k R / 2)^n / n! is below 1e-16
+  int nleaf, D, p, nmin;                 // nmin: order from which (k R / 2)^n / n! is below 1e-18
   double d, R, far2;                     // leaf side, radius, squared distance from which a leaf is far
   const int *ne, *bb, *be;
   const double2* ctr;
@@ -3084,7 +3144,6 @@ __global__ void leaf_lengths_kernel(int nleaf, const int* __restrict__ ne, const
   hr[i] = double2{lo, hi};
 }
 
-template <bool WU, bool WD>
 __global__ void __launch_bounds__(FL_NT) field_leaf_kernel(
     const __grid_constant__ FieldLeaf fl, int npts, const double2* __restrict__ pts, int nsl, double k, double eta,
     double H, double ox, double oy, double x0, double y0, int mdir, cplx alpha, const double2* __restrict__ sc,
@@ -3097,12 +3156,12 @@ __global__ void __launch_bounds__(FL_NT) field_leaf_kernel(
     return;
   }
   __shared__ int s_li[FL_CAP], s_img[FL_CAP], s_off[FL_CAP + 1], s_n;
-  __shared__ cplx s_red[2][FL_NT / 32];
+  __shared__ cplx s_red[FL_NT / 32];
   const int tid = threadIdx.x, lane = tid & 31, pi = blockIdx.x / nsl, sl = blockIdx.x - pi * nsl;
   const int nim = 2 * mdir + 1, jobs = fl.nleaf * nim, P = 2 * fl.p + 1;
   double2 x = pts[pi];
   x.y -= floor((x.y - y0) / H) * H;
-  cplx acc{0, 0}, dacc{0, 0};
+  cplx dacc{0, 0};
   if (tid == 0) s_n = 0;
   __syncthreads();
   for (int base = sl * FL_NT; base < jobs; base += nsl * FL_NT) {
@@ -3124,13 +3183,9 @@ __global__ void __launch_bounds__(FL_NT) field_leaf_kernel(
         for (int q = 2; q <= 4; ++q)
           if (lo >= c_glthr[0][q] * hr.y && hi < c_glthr[0][q - 1] * hr.x) g = q;
       if (g) {
-        const int q = (int)ceilf(15.2f / log10f((float)(r / (fl.R + 0.5 * hr.y))));
-        cplx u, du;
-        multipole_eval<WU, WD>(k, vx, vy, fl.p, min(fl.p, max(fl.nmin, q)), nullptr,
-                               fl.M + ((size_t)(g - 2) * fl.nleaf + li) * P, u, du);
-        const cplx ph = ipow_phase(alpha, m);
-        if (WU) acc += ph * u;
-        if (WD) dacc += ph * du;
+        const int q = (int)ceilf(18.0f / log10f((float)(r / (fl.R + 0.5 * hr.y))));
+        dacc += ipow_phase(alpha, m) * multipole_dx1(k, vx, vy, fl.p, min(fl.p, max(fl.nmin, q)), nullptr,
+                                                     fl.M + ((size_t)(g - 2) * fl.nleaf + li) * P);
       } else {
         const int o = atomicAdd(&s_n, 1);          // below FL_CAP: a list of more than FL_CAP - FL_NT was emptied
         s_li[o] = li;
@@ -3172,29 +3227,20 @@ __global__ void __launch_bounds__(FL_NT) field_leaf_kernel(
         const double q = sqrt((x.x - c.x) * (x.x - c.x) + (x.y - c.y) * (x.y - c.y)) / hh;
         cplx S{0, 0}, Dv{0, 0}, K{0, 0}, T{0, 0};
         pair4_f64(k, x, nx, c, st[f], snu[f], hh, gl_order(q, 0), S, Dv, K, T);
-        const cplx ph = ipow_phase(alpha, m);
-        if (WU) acc += ph * (Dv * dens[2 * f] - eta * mul_i(S * dens[2 * f + 1]));
-        if (WD) dacc += ph * (T * dens[2 * f] - eta * mul_i(K * dens[2 * f + 1]));
+        dacc += ipow_phase(alpha, m) * (T * dens[2 * f] - eta * mul_i(K * dens[2 * f + 1]));
       }
       __syncthreads();
       if (tid == 0) s_n = 0;
     }
     __syncthreads();
   }
-  if (WU) acc = warp_sum(acc);
-  if (WD) dacc = warp_sum(dacc);
-  if (lane == 0) {
-    s_red[0][tid >> 5] = acc;
-    s_red[1][tid >> 5] = dacc;
-  }
+  dacc = warp_sum(dacc);
+  if (lane == 0) s_red[tid >> 5] = dacc;
   __syncthreads();
   if (tid == 0) {
-    for (int i = 1; i < FL_NT / 32; ++i) {
-      acc += s_red[0][i];
-      dacc += s_red[1][i];
-    }
+    for (int i = 1; i < FL_NT / 32; ++i) dacc += s_red[i];
     cplx* o = part + 2 * ((size_t)pi * (nsl + 1) + sl);
-    o[0] = acc;
+    o[0] = cplx{0, 0};
     o[1] = dacc;
   }
 }
@@ -3208,7 +3254,7 @@ static bool field_leaf(const pfmbem* h, int npts, FieldLeaf& fl) {
   fl.R = (h->tree == 1 ? 0.5 : 0.5 * sqrt(2.0)) * L.d;
   const double kd = 2.0 * h->k * fl.R;
   if (kd < 1e-6 || L.p < 20 || L.p < kd + 1.8 * pow(10.0, 2.0 / 3.0) * cbrt(kd)) return false;
-  const double far = (fl.R + 0.5 * h->hmax) / fmin(0.26, pow(10.0, -14.7 / (L.p + 1)));
+  const double far = (fl.R + 0.5 * h->hmax) / fmin(0.26, pow(10.0, -18.0 / (L.p + 1)));
   fl.far2 = far * far;
   fl.nleaf = L.nne;
   fl.D = h->D;
@@ -3219,7 +3265,7 @@ static bool field_leaf(const pfmbem* h, int npts, FieldLeaf& fl) {
   fl.be = L.box_end;
   fl.ctr = L.ctr;
   double t = 1.0;
-  for (fl.nmin = 0; fl.nmin < L.p && t > 1e-16; ++fl.nmin) t *= 0.25 * kd / (fl.nmin + 1);
+  for (fl.nmin = 0; fl.nmin < L.p && t > 1e-18; ++fl.nmin) t *= 0.25 * kd / (fl.nmin + 1);
   return true;
 }
 
@@ -3286,16 +3332,26 @@ cudaError_t k_field(pfmbem* h, int npts, const double2* pts, cplx* u, cplx* dudx
   FieldTree ft;
   const bool tree = by_tree && !u && field_tree(h, ft);
   FieldLeaf fl;
-  const bool leaf = !tree && field_leaf(h, npts, fl);
+  bool leaf = !tree && !u && field_leaf(h, npts, fl);
   // slices of a point's sum: about 32 warps per SM in all, at least 8 terms a lane; by
   // leaves about eight blocks per SM, at least a pair a thread
-  const int64_t terms = (int64_t)(2 * mdir + 1) * (leaf ? fl.nleaf : h->E);
-  const int nsl = tree ? 1
-                       : (int)std::max<int64_t>(1, leaf ? std::min<int64_t>((152 * 8 + npts - 1) / npts, terms / FL_NT)
-                                                        : std::min<int64_t>((152 * 32 + npts - 1) / npts, terms / 256));
+  auto slices = [&]() -> int {
+    if (tree || u) return 1;      // u: one order of its sum (field_direct_kernel)
+    const int64_t terms = (int64_t)(2 * mdir + 1) * (leaf ? fl.nleaf : h->E);
+    return (int)std::max<int64_t>(1, std::min<int64_t>((152 * (leaf ? 8 : 32) + npts - 1) / npts, terms / 256));
+  };
+  int nsl = slices();
   void* buf = nullptr;
-  const size_t npart = 2 * (size_t)npts * (nsl + 1), nrule = leaf ? 3 * (size_t)fl.nleaf * (2 * fl.p + 1) : 0;
+  size_t npart = 2 * (size_t)npts * (nsl + 1);
+  const size_t nrule = leaf ? 3 * (size_t)fl.nleaf * (2 * fl.p + 1) : 0;
   cudaError_t e = cudaMallocAsync(&buf, sizeof(cplx) * (npart + nrule + (leaf ? fl.nleaf : 0)), h->stream);
+  if (e == cudaErrorMemoryAllocation && leaf) {     // no room for the multipoles: element by element
+    cudaGetLastError();
+    leaf = false;
+    nsl = slices();
+    npart = 2 * (size_t)npts * (nsl + 1);
+    e = cudaMallocAsync(&buf, sizeof(cplx) * npart, h->stream);
+  }
   if (e != cudaSuccess) return e;
   cplx* part = static_cast<cplx*>(buf);
   prof_begin(h, PH_OUT);
@@ -3305,14 +3361,9 @@ cudaError_t k_field(pfmbem* h, int npts, const double2* pts, cplx* u, cplx* dudx
         h->dens, p0, w0, L0, part);
   } else if (leaf) {
     field_rules(h, fl, part + npart, reinterpret_cast<double2*>(part + npart + nrule));
-    auto launch = [&](auto kern) {
-      kern<<<npts * nsl + (npts + FL_NT - 1) / FL_NT, FL_NT, 0, h->stream>>>(
-          fl, npts, pts, nsl, h->k, h->eta, h->H, ox, oy, h->x0, h->y0, mdir, h->alpha, h->s_c, h->s_t, h->s_nu,
-          h->s_h, h->dens, p0, w0, L0, part);
-    };
-    if (u && dudx1) launch(field_leaf_kernel<true, true>);
-    else if (u) launch(field_leaf_kernel<true, false>);
-    else launch(field_leaf_kernel<false, true>);
+    field_leaf_kernel<<<npts * nsl + (npts + FL_NT - 1) / FL_NT, FL_NT, 0, h->stream>>>(
+        fl, npts, pts, nsl, h->k, h->eta, h->H, ox, oy, h->x0, h->y0, mdir, h->alpha, h->s_c, h->s_t, h->s_nu, h->s_h,
+        h->dens, p0, w0, L0, part);
   } else {
     const unsigned grid = (unsigned)(((int64_t)npts * nsl + 3) / 4 + (npts + 127) / 128);
     auto launch = [&](auto kern) {

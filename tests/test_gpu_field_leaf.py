@@ -1,4 +1,4 @@
-"""Field and derivative by the leaves' multipoles (32 points and more) against the direct
+"""The field's derivative by the leaves' multipoles (32 points and more) against the direct
 sums (fewer points in a call) on the same handle: square and triangle trees, blocks wider
 than their period, fibers of unequal elements, deep trees, on-the-fly handles, long
 wavelengths, densities that radiate and that cancel."""
@@ -62,13 +62,12 @@ def test_leaves_match_direct_sums(w, opts, smooth):
         psi[0::2] = np.exp(1j * w.k * (c @ dr))
         psi[1::2] = psi[0::2] * ((np.stack([d[:, 1], -d[:, 0]], axis=1) / h[:, None]) @ dr)
     pts = points(w, 75)
-    u, du = np.zeros(75, np.complex128), np.zeros(75, np.complex128)
-    pf.pfmbem_field_dx1(s.h, psi, pts, u, du)
+    du = np.zeros(75, np.complex128)
+    pf.pfmbem_field_dx1(s.h, psi, pts, None, du)
     r = 0.2 * float(np.min(w.radii))
     q = np.sum(h * np.abs(psi[0::2])), np.sum(h * np.abs(psi[1::2])) * w.k
     for i in range(0, 75, 25):
-        v, dv = np.zeros(25, np.complex128), np.zeros(25, np.complex128)
-        pf.pfmbem_field_dx1(s.h, psi, np.ascontiguousarray(pts[i:i + 25]), v, dv)
-        assert np.max(np.abs(u[i:i + 25] - v)) < 1e-13 * (q[0] * (w.k + 1 / r) + q[1])
+        dv = np.zeros(25, np.complex128)
+        pf.pfmbem_field_dx1(s.h, psi, np.ascontiguousarray(pts[i:i + 25]), None, dv)
         assert np.max(np.abs(du[i:i + 25] - dv)) < 1e-13 * (q[0] * (w.k + 1 / r) ** 2 + q[1] * (w.k + 1 / r))
     s.close()
