@@ -2724,7 +2724,7 @@ pfmbem_status field_points(pfmbem* h, const double* psi, int npts, const double*
   cplx* ud = dalloc_tmp<cplx>(h, 2 * (size_t)npts);
   if (!pd || !ud) return fail(h, PFMBEM_ENOMEM, "field buffers");
   CK(cudaMemcpyAsync(pd, hp.data(), sizeof(double2) * npts, cudaMemcpyHostToDevice, h->stream));
-  CK(k_field_prepare(h, psid));
+  CK(k_field_prepare(h, psid, u != nullptr));
   CK(k_field(h, npts, pd, u ? ud : nullptr, du ? ud + npts : nullptr, by_tree));
   if (u)
     CK(cudaMemcpyAsync(u, ud, sizeof(cplx) * npts, is_device_ptr(u) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,

@@ -409,7 +409,7 @@ cudaError_t k_warm_features(pfmbem* h, float* x_dev);
 cudaError_t k_warm_features_local(pfmbem* h, int K, float* x_dev);
 cudaError_t k_warm_targets(pfmbem* h, int nm, const cplx* psi, float* t_dev);
 cudaError_t k_warm_decode(pfmbem* h, int nm, const float* y_dev, cplx* psi);
-cudaError_t k_field_prepare(pfmbem* h, const cplx* psi);
+cudaError_t k_field_prepare(pfmbem* h, const cplx* psi, bool with_u);
 cudaError_t k_coefficients(pfmbem* h, const cplx* psi, int norders, const int* orders_host, cplx* out_dev);
 
 // ------------------------------------------------------------ kernel launches

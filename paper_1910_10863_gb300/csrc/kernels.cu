@@ -1038,16 +1038,18 @@ __global__ void p2m_f64_kernel(const int* __restrict__ ne, const int* __restrict
 // ---------------------------------------------------------------- M2M (FP64)
 // M(parent) = sum_children A_q M(child), A_q[n][m] = J^-_{n-m}(k(O_child - O_parent)) w^c_m / w^p_n.
 // Children nch box + q, q < nch; the child's operator is q, or aidx[child] where
-// the children's offsets vary (triangle tree).  M2M_SPLIT groups of 64 threads
+// the children's offsets vary (triangle tree).  SPLIT groups of 64 threads
 // share the children's coefficients: one thread's chain of 4 Pc operator loads
-// was the kernel's time (the block has little else to overlap it with).
+// is the kernel's time (the block has little else to overlap it with).  Four of
+// them, M2M_SPLIT, but for the field u, whose sums keep one order (upward_f64).
 constexpr int M2M_SPLIT = 4;
-__global__ void __launch_bounds__(64 * M2M_SPLIT) m2m_f64_kernel(const int* __restrict__ ne, int P, int Pc, const cplx* __restrict__ A,
-                               const int* __restrict__ cbb, const int* __restrict__ cbe,
-                               const cplx* __restrict__ Mc, cplx* __restrict__ Mp, int nch,
-                               const int* __restrict__ aidx) {
+template <int SPLIT>
+__global__ void __launch_bounds__(64 * SPLIT) m2m_f64_kernel(
+    const int* __restrict__ ne, int P, int Pc, const cplx* __restrict__ A, const int* __restrict__ cbb,
+    const int* __restrict__ cbe, const cplx* __restrict__ Mc, cplx* __restrict__ Mp, int nch,
+    const int* __restrict__ aidx) {
   const int box = ne[blockIdx.x];
-  __shared__ cplx sm[6 * PF_NCOEF], red[M2M_SPLIT][64];
+  __shared__ cplx sm[6 * PF_NCOEF], red[SPLIT][64];
   for (int i = threadIdx.x; i < nch * Pc; i += blockDim.x) sm[i] = Mc[(size_t)nch * box * Pc + i];
   __syncthreads();
   const int part = threadIdx.x >> 6, lane = threadIdx.x & 63;
@@ -1061,12 +1063,16 @@ __global__ void __launch_bounds__(64 * M2M_SPLIT) m2m_f64_kernel(const int* __re
       const cplx* col = A + (size_t)op * Pc * P + n;              // transposed [op][m][n]
       const cplx* mc = sm + q * Pc;
 #pragma unroll 4
-      for (int m = part; m < Pc; m += M2M_SPLIT) acc += col[(size_t)m * P] * mc[m];
+      for (int m = part; m < Pc; m += SPLIT) acc += col[(size_t)m * P] * mc[m];
+    }
+    if (SPLIT == 1) {
+      if (n < P) Mp[(size_t)box * P + n] = acc;
+      continue;
     }
     red[part][lane] = acc;
     __syncthreads();
     if (part == 0 && n < P) {
-      for (int i = 1; i < M2M_SPLIT; ++i) acc += red[i][lane];
+      for (int i = 1; i < SPLIT; ++i) acc += red[i][lane];
       Mp[(size_t)box * P + n] = acc;
     }
     __syncthreads();
@@ -2425,7 +2431,11 @@ cudaError_t k_build_fmm_caches(pfmbem* h) {
 // triangles' centroids and M2M up to the hexagonal cells (six children each at
 // level 0); their local expansions come from the operator between the cells
 // (top_apply_kernel, in the product).
-static void upward_f64(pfmbem* h, const cplx* x) {
+// one_sum (the field u): the multipoles by the elements' integrals and M2M in one sum a
+// coefficient.  Where a density radiates almost nothing, the field from the far images
+// is what other terms of the size of 1 cancel to 1e-8, and the cached coefficients and
+// M2M in shares, each as accurate, moved u by 1e-9 to 6e-9 of itself.
+static void upward_f64(pfmbem* h, const cplx* x, bool one_sum = false) {
   cudaStream_t st = h->stream;
   const int E = h->E, D = h->D;
   prof_begin(h, PH_GATHER);
@@ -2433,7 +2443,7 @@ static void upward_f64(pfmbem* h, const cplx* x) {
   prof_end(h, PH_GATHER);
   Level& leaf = h->lev[D];
   prof_begin(h, PH_P2M);
-  if (h->cached || h->tri_cache)       // the coefficients are there
+  if ((h->cached || h->tri_cache) && !one_sum)       // the coefficients are there
     p2m_apply_t_kernel<cplx><<<leaf.nne, round32(leaf.P), 0, st>>>(leaf.ne, leaf.box_begin, leaf.box_end, leaf.P,
                                                                    h->p2m_c, h->dens, leaf.M);
   else
@@ -2445,8 +2455,12 @@ static void upward_f64(pfmbem* h, const cplx* x) {
     Level& a = h->lev[l];
     Level& c = h->lev[l + 1];
     prof_begin(h, PH_M2M);
-    m2m_f64_kernel<<<a.nne, 64 * M2M_SPLIT, 0, st>>>(a.ne, a.P, c.P, a.m2m, c.box_begin, c.box_end, c.M, a.M,
-                                                   h->tree == 1 && l == 0 ? 6 : 4, c.pidx);
+    const int nch = h->tree == 1 && l == 0 ? 6 : 4;
+    if (one_sum)
+      m2m_f64_kernel<1><<<a.nne, 64, 0, st>>>(a.ne, a.P, c.P, a.m2m, c.box_begin, c.box_end, c.M, a.M, nch, c.pidx);
+    else
+      m2m_f64_kernel<M2M_SPLIT><<<a.nne, 64 * M2M_SPLIT, 0, st>>>(a.ne, a.P, c.P, a.m2m, c.box_begin, c.box_end, c.M,
+                                                                  a.M, nch, c.pidx);
     prof_end(h, PH_M2M);
   }
   if (h->tree == 1) return;
@@ -2568,8 +2582,8 @@ static cudaError_t matvec_tri_cached(pfmbem* h, const cplx* x, cplx* y) {
       e = k_tri_m2m_dd(h, l);
       if (e != cudaSuccess) return e;
     } else {
-      m2m_f64_kernel<<<a.nne, 64 * M2M_SPLIT, 0, st>>>(a.ne, a.P, c.P, a.m2m, c.box_begin, c.box_end, c.M, a.M,
-                                                     l == 0 ? 6 : 4, c.pidx);
+      m2m_f64_kernel<M2M_SPLIT><<<a.nne, 64 * M2M_SPLIT, 0, st>>>(a.ne, a.P, c.P, a.m2m, c.box_begin, c.box_end, c.M,
+                                                                  a.M, l == 0 ? 6 : 4, c.pidx);
     }
     prof_end(h, PH_M2M);
   }
@@ -3308,8 +3322,9 @@ static bool field_tree(const pfmbem* h, FieldTree& ft) {
   return true;
 }
 
-cudaError_t k_field_prepare(pfmbem* h, const cplx* psi) {
-  upward_f64(h, psi);
+// with_u: the field itself is asked for (upward_f64's one_sum).
+cudaError_t k_field_prepare(pfmbem* h, const cplx* psi, bool with_u) {
+  upward_f64(h, psi, with_u);
   if (h->tree == 1) {
     // the super root's local expansion of the images |m| >= m0
     prof_begin(h, PH_LOCAL);
