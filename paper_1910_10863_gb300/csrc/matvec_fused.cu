@@ -3623,14 +3623,16 @@ cudaError_t k_tri_top(pfmbem* h, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// The limits of the dynamic shared memory belong to the kernel, not to the handle: both
+// are set to the most that any handle takes, so that handles of other sizes in other
+// threads never lower them between this call's setting and its launch.
 cudaError_t k_tri_fiber(pfmbem* h, const cplx* x, cplx* y, cudaStream_t st) {
-  const size_t smem = sizeof(float4) * 3 * 2 * (size_t)h->max_fiber;
-  if (smem > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(tri_fiber_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  tri_fiber_kernel<<<h->nchunk, 256, smem, st>>>(h->fb_chunk, h->fib_off, h->fb_base, h->fb_val, x, y, h->fb_circ);
+  constexpr size_t per = sizeof(float4) * 3 * 2;
+  const cudaError_t e = cudaFuncSetAttribute(tri_fiber_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(per * TRI_FIBER_MAX));
+  if (e != cudaSuccess) return e;
+  tri_fiber_kernel<<<h->nchunk, 256, per * h->max_fiber, st>>>(h->fb_chunk, h->fib_off, h->fb_base, h->fb_val, x, y,
+                                                               h->fb_circ);
   return cudaGetLastError();
 }
 
@@ -3707,10 +3709,10 @@ cudaError_t k_tri_m2l_dd(pfmbem* h) {
     smem = std::max(smem, k_tri_m2l_smem(L.P));
   }
   if (a.n == 0) return cudaSuccess;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(tri_m2l_dd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  // (the limit as in k_tri_fiber)
+  const cudaError_t e =
+      cudaFuncSetAttribute(tri_m2l_dd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRI_M2L_SMEM);
+  if (e != cudaSuccess) return e;
   tri_m2l_dd_kernel<<<a.first[a.n], 256, smem, h->stream>>>(a, h->alpha);
   return cudaGetLastError();
 }

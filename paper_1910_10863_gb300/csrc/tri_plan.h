@@ -390,7 +390,7 @@ static pfmbem_status build_plan_tri(pfmbem* h, const double* nodes, const std::v
                          2.0 * E * 2 * h->lev[D].P * sizeof(cplx);
     // (the near-field build's shared memory: per-source and per-target arrays)
     const size_t nb_smem = sizeof(int) * (13 * (size_t)h->nc_maxns + 4 * (size_t)h->leaf_maxn + 16);
-    h->tri_cache = h->opt.near_mode == 0 && h->max_fiber <= 1024 && bytes < 0.5 * (double)freeb &&
+    h->tri_cache = h->opt.near_mode == 0 && h->max_fiber <= TRI_FIBER_MAX && bytes < 0.5 * (double)freeb &&
                    nb_smem <= 200 * 1024;
   }
   if (h->tri_cache) {
