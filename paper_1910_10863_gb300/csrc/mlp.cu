@@ -32,7 +32,6 @@ struct pfmbem_mlp {
   float* dB = nullptr;
   float* tgt = nullptr;            // a host batch's targets
   float* loss = nullptr;           // device scalar
-  float* hloss = nullptr;          // page-locked: the loss read back
 };
 
 namespace {
@@ -589,7 +588,7 @@ pfmbem_status pfmbem_mlp_create(int in, int hidden, int layers, int out, uint64_
   cudaMemsetAsync(m->m2, 0, off * sizeof(float), m->stream);
   cudaStreamSynchronize(m->stream);
   cudaFree(fan_d);
-  if (cudaMalloc(&m->loss, sizeof(float)) != cudaSuccess || cudaMallocHost(&m->hloss, sizeof(float)) != cudaSuccess) {
+  if (cudaMalloc(&m->loss, sizeof(float)) != cudaSuccess) {
     pfmbem_mlp_destroy(m);
     return PFMBEM_ENOMEM;
   }
@@ -614,7 +613,6 @@ void pfmbem_mlp_destroy(pfmbem_mlp_t m) {
   cudaFree(m->dA);
   cudaFree(m->dB);
   cudaFree(m->tgt);
-  cudaFreeHost(m->hloss);
   delete m;
 }
 
@@ -685,10 +683,9 @@ pfmbem_status pfmbem_mlp_train(pfmbem_mlp_t m, int B, const float* X, const floa
       cudaMemcpyAsync(grad, g, m->nparams * sizeof(float),
                       is_dev(grad) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
     return PFMBEM_ECUDA;
-  if (loss && cudaMemcpyAsync(m->hloss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
+  if (loss && cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
     return PFMBEM_ECUDA;
   if (cudaStreamSynchronize(m->stream) != cudaSuccess) return PFMBEM_ECUDA;
-  if (loss) *loss = *m->hloss;
   return cudaGetLastError() == cudaSuccess ? PFMBEM_OK : PFMBEM_ECUDA;
 }
 
