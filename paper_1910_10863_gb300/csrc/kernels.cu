@@ -14,6 +14,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "side_chain.h"
 
 // Gauss-Legendre rules g = 1..16 on [-1, 1]: node q of rule g at [g-1][q].
 __constant__ double c_glx[PF_GLMAX][PF_GLMAX];
@@ -2542,16 +2543,12 @@ cudaError_t k_near64(pfmbem* h) {
 // (which adds to y) wait for that stream.  So M2L comes before L2L and adds
 // to expansions that the upward pass cleared.  16384 elements, p = 30: 1.78 ms as
 // one chain.
-static cudaError_t matvec_tri_cached(pfmbem* h, const cplx* x, cplx* y) {
-  cudaStream_t st = h->stream;
+static cudaError_t tri_chains(pfmbem* h, const cplx* x, cplx* y, bool fork) {
+  cudaStream_t st = h->stream, st2 = fork ? h->aux[0] : st;
   const int E = h->E, D = h->D;
   Level& leaf = h->lev[D];
   const cplx alpha = h->alpha;
-  cudaError_t e = k_near64(h);
-  if (e != cudaSuccess) return e;
-  // one chain where phases are timed, for their events lie on one stream
-  const bool fork = h->aux[0] && h->aux_ev[0] && h->fork_ev && h->side_ev && !h->prof.on;
-  cudaStream_t st2 = fork ? h->aux[0] : st;
+  cudaError_t e = cudaSuccess;
   prof_begin(h, PH_GATHER);
   gather_dens_kernel<<<(E + 255) / 256, 256, 0, st>>>(E, h->s_perm, h->s_ph, x, h->dens);
   prof_end(h, PH_GATHER);
@@ -2632,6 +2629,15 @@ static cudaError_t matvec_tri_cached(pfmbem* h, const cplx* x, cplx* y) {
   if ((e = k_tri_l2p(h, y)) != cudaSuccess) return e;
   prof_end(h, PH_L2P);
   return cudaGetLastError();
+}
+
+static cudaError_t matvec_tri_cached(pfmbem* h, const cplx* x, cplx* y) {
+  cudaError_t e = k_near64(h);
+  if (e != cudaSuccess) return e;
+  // one chain where phases are timed, for their events lie on one stream
+  const bool fork = h->aux[0] && h->aux_ev[0] && h->fork_ev && h->side_ev && !h->prof.on;
+  if (!fork) return tri_chains(h, x, y, false);
+  return run_with_side(h->stream, h->aux[0], h->aux_ev[0], [&] { return tri_chains(h, x, y, true); });
 }
 
 cudaError_t k_tri_caches(pfmbem* h) {
