@@ -456,7 +456,6 @@ cudaError_t k_tri_m2l_dd(pfmbem* h);
 size_t k_tri_m2l_smem(int P);
 constexpr int TRI_FIBER_MAX = 1024;           // most elements of a fiber with cached tables
 constexpr size_t TRI_M2L_SMEM = 200 * 1024;   // above it a level's M2L goes target by target
-cudaError_t k_tri_words(pfmbem* h);
 cudaError_t k_tri_top(pfmbem* h, cudaStream_t st);
 cudaError_t k_tri_fiber(pfmbem* h, const cplx* x, cplx* y, cudaStream_t st);
 cudaError_t k_tri_l2p(pfmbem* h, cplx* y);

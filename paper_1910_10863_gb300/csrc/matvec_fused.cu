@@ -3485,45 +3485,70 @@ static dim3 tri_block(int P, int shares) {
   return dim3(x, std::max(1, std::min(shares, 1024 / x)));
 }
 
-// ------------------------------------- triangle tree: tables as double-float words
-// n FP64 values turned into the words of their hi and lo parts where they lie.
-__global__ void dd_words_kernel(size_t n, cplx* a) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const cplx v = a[i];
-    reinterpret_cast<float4*>(a)[i] = dd_word(v);
-  }
+// ------------------------------------------------ triangle tree: FP64 sums of tables
+// The operator between the cells, the same-fiber rows and L2P are sums of table entries in
+// FP64, as accurate as the tables: with table and vector as double-float words the product's
+// rounding was 2e-14 to 6e-14 of its result, with these sums 0.9e-15 to 1.8e-15 (x against
+// x (1 + 2^-26), nine blocks).  The first two run beside the M2M and M2L; the product takes
+// 1020 us on the 8x8 hexagon block (16384 elements, p = 30), 1765 as one chain, 910 with the words.
+__device__ __forceinline__ cplx ld2(const cplx* p) {       // 16 bytes; the tables are aligned to them
+  const double2 v = __ldcs(reinterpret_cast<const double2*>(p));
+  return cplx{v.x, v.y};
+}
+// acc += a b in four FP64 instructions (the pipe that bounds these sums; the operators of
+// cplx take six: the product is rounded before it is added)
+__device__ __forceinline__ void cmac(cplx& acc, cplx a, cplx b) {
+  acc.re = fma(a.re, b.re, acc.re);
+  acc.im = fma(a.re, b.im, acc.im);
+  acc.re = fma(-a.im, b.im, acc.re);
+  acc.im = fma(a.im, b.re, acc.im);
+}
+// Sums over the warp of four values, halved between the lanes in the first two steps
+// (six additions instead of twenty): lanes 0, 8, 16, 24 hold the sums of a, b, c, d.
+__device__ __forceinline__ double wsum4(double a, double b, double c, double d, int lane) {
+  const bool u = (lane & 16) != 0, v = (lane & 8) != 0;
+  const double p = (u ? c : a) + __shfl_xor_sync(0xffffffffu, u ? a : c, 16);
+  const double q = (u ? d : b) + __shfl_xor_sync(0xffffffffu, u ? b : d, 16);
+  double r = (v ? q : p) + __shfl_xor_sync(0xffffffffu, v ? p : q, 8);
+  r += __shfl_xor_sync(0xffffffffu, r, 4);
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  return r + __shfl_xor_sync(0xffffffffu, r, 1);
 }
 
-// The operator between the cells, L0 = TOP M0 (the words of TOP [rows][rows]): one
-// warp per row, the multipoles as words in shared memory, a tile of TRI_TILE at a
-// time.  Bound by the read of TOP; in FP64 instructions their pipe bound it (213 us
-// for 3904 rows, 244 MB).
+// L0 = TOP M0, TOP [rows][rows]: one warp per row, the multipoles in shared memory, a tile
+// of TRI_TILE at a time.  Bound by the FP64 pipe: 3904 rows (244 MB) take 141 us.
 constexpr int TRI_TILE = 1024;
-__global__ void __launch_bounds__(256) tri_top_kernel(int rows, const float4* __restrict__ TOP,
+__global__ void __launch_bounds__(256) tri_top_kernel(int rows, const cplx* __restrict__ TOP,
                                                       const cplx* __restrict__ M0, cplx* __restrict__ L0) {
-  __shared__ float4 sw[TRI_TILE];
+  __shared__ __align__(16) cplx sw[TRI_TILE];
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const float4* t = TOP + (size_t)min(row, rows - 1) * rows;
-  dflt re{0, 0}, im{0, 0};
+  const cplx* t = TOP + (size_t)min(row, rows - 1) * rows;
+  cplx a{0, 0}, b{0, 0}, c{0, 0}, d{0, 0};
   for (int c0 = 0; c0 < rows; c0 += TRI_TILE) {
     const int nc = min(TRI_TILE, rows - c0);
     __syncthreads();
-    for (int i = threadIdx.x; i < nc; i += 256) sw[i] = dd_word(M0[c0 + i]);
+    for (int i = threadIdx.x; i < nc; i += 256) sw[i] = M0[c0 + i];
     __syncthreads();
-#pragma unroll 4
-    for (int i = lane; i < nc; i += 32) dd_cmac(re, im, __ldcs(t + c0 + i), sw[i]);
+    int i = lane;
+    for (; i + 96 < nc; i += 128) {
+      const cplx t0 = ld2(t + c0 + i), t1 = ld2(t + c0 + i + 32), t2 = ld2(t + c0 + i + 64), t3 = ld2(t + c0 + i + 96);
+      cmac(a, t0, sw[i]);
+      cmac(b, t1, sw[i + 32]);
+      cmac(c, t2, sw[i + 64]);
+      cmac(d, t3, sw[i + 96]);
+    }
+    for (; i < nc; i += 32) cmac(a, ld2(t + c0 + i), sw[i]);
   }
-  const dflt r = dd_wsum(re), q = dd_wsum(im);
-  if (lane == 0 && row < rows) L0[row] = cplx{dd_value(r), dd_value(q)};
+  a = wsum((a + b) + (c + d));
+  if (lane == 0 && row < rows) L0[row] = a;
 }
 
 // Same-fiber rows of the triangle tree's cached product, y = B x by chunks of rows of a
 // fiber (chunk: fiber, first and last row).  A circulant fiber's generating row pair
-// and x are staged as words and a warp sums a row pair with x rotated by 2e, sum_c
-// R[(c - 2e) mod 2N] x[c] = sum_c R[c] x[(c + 2e) mod 2N]; the rows of another fiber
-// are FP64 sums over its table (converting a word costs what it saves there).  FP64
-// sums and the division by the phase in one lane kept the FP64 pipe busy for 299 us
-// at 64 circulant fibers of 256 elements.
+// and x lie in shared memory and a warp sums a row pair with x rotated by 2e, sum_c
+// R[(c - 2e) mod 2N] x[c] = sum_c R[c] x[(c + 2e) mod 2N]; another fiber's rows are read
+// from its table.  Bound by the FP64 pipe: 64 circulant fibers of 256 elements take 125 us
+// (301 with the row pair read from the table and the phase divided out in one lane).
 __global__ void __launch_bounds__(256) tri_fiber_kernel(const int* __restrict__ chunk, const int* __restrict__ foff,
                                                         const int64_t* __restrict__ fbase,
                                                         const cplx* __restrict__ val, const cplx* __restrict__ x,
@@ -3533,28 +3558,36 @@ __global__ void __launch_bounds__(256) tri_fiber_kernel(const int* __restrict__ 
   const int f0 = foff[fb], n2 = 2 * (foff[fb + 1] - f0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const cplx* B = val + fbase[fb];
+  cplx *xs = reinterpret_cast<cplx*>(tri_sm), *rw = xs + n2;      // x, the row pair
+  for (int i = threadIdx.x; i < n2; i += blockDim.x) xs[i] = x[2 * f0 + i];
   if (circ[fb]) {
-    float4 *xw = tri_sm, *rw = tri_sm + n2;              // x, the row pair
-    for (int i = threadIdx.x; i < n2; i += blockDim.x) xw[i] = dd_word(x[2 * f0 + i]);
-    for (int i = threadIdx.x; i < 2 * n2; i += blockDim.x) rw[i] = dd_word(B[i]);
+    for (int i = threadIdx.x; i < 2 * n2; i += blockDim.x) rw[i] = B[i];
     __syncthreads();
     for (int r = rb + 2 * warp; r < re; r += 2 * nw) {   // chunks hold whole row pairs
-      dflt a{0, 0}, b{0, 0}, c{0, 0}, d{0, 0};
-#pragma unroll 2
-      for (int i = lane; i < n2; i += 32) {
-        int j = i + r;
+      cplx a{0, 0}, b{0, 0}, c{0, 0}, d{0, 0};
+      int i = lane;
+      for (; i + 32 < n2; i += 64) {
+        int j = i + r, k = i + 32 + r;
         if (j >= n2) j -= n2;
-        const float4 v = xw[j];
-        dd_cmac(a, b, rw[i], v);
-        dd_cmac(c, d, rw[n2 + i], v);
+        if (k >= n2) k -= n2;
+        const cplx v = xs[j], w = xs[k];
+        cmac(a, rw[i], v);
+        cmac(b, rw[n2 + i], v);
+        cmac(c, rw[i + 32], w);
+        cmac(d, rw[n2 + i + 32], w);
       }
-      const dflt s = dd_wsum4(a, b, c, d, lane);         // lanes 0, 8, 16, 24
-      if ((lane & 7) == 0) reinterpret_cast<double*>(y + 2 * f0 + r)[lane >> 3] = dd_value(s);
+      if (i < n2) {
+        const cplx v = xs[i + r < n2 ? i + r : i + r - n2];
+        cmac(a, rw[i], v);
+        cmac(b, rw[n2 + i], v);
+      }
+      a += c;
+      b += d;
+      const double s = wsum4(a.re, a.im, b.re, b.im, lane);         // lanes 0, 8, 16, 24
+      if ((lane & 7) == 0) reinterpret_cast<double*>(y + 2 * f0 + r)[lane >> 3] = s;
     }
     return;
   }
-  cplx* xs = reinterpret_cast<cplx*>(tri_sm);
-  for (int i = threadIdx.x; i < n2; i += blockDim.x) xs[i] = x[2 * f0 + i];
   __syncthreads();
   for (int r = rb + warp; r < re; r += nw) {
     const cplx* row = B + (int64_t)r * n2;
@@ -3562,10 +3595,10 @@ __global__ void __launch_bounds__(256) tri_fiber_kernel(const int* __restrict__ 
     int c = lane;
     for (; c + 32 < n2; c += 64) {
       const cplx r0 = row[c], r1 = row[c + 32];
-      a += r0 * xs[c];
-      b += r1 * xs[c + 32];
+      cmac(a, r0, xs[c]);
+      cmac(b, r1, xs[c + 32]);
     }
-    if (c < n2) a += row[c] * xs[c];
+    if (c < n2) cmac(a, row[c], xs[c]);
     a = wsum(a + b);
     if (lane == 0) y[2 * f0 + r] = a;
   }
@@ -3573,13 +3606,13 @@ __global__ void __launch_bounds__(256) tri_fiber_kernel(const int* __restrict__ 
 
 // L2P and the near sums (U, already there), added to y in the caller's order:
 // y_e += alpha^{m0} (U + U', c2 (dU + dU')), U'_s = sum_l c[s][0][l] L_l, dU'_s =
-// sum_l c[s][1][l] L_l with the words of c, an element's 2 P words together.  A warp
-// per element; one warp of the block does the FP64 ends of its eight elements (a warp
-// instruction of the FP64 pipe costs the same for one lane as for sixteen).  With the
-// coefficients element by element (16 bytes of each line for a leaf of one) 16384
-// elements took 78 to 134 us.
+// sum_l c[s][1][l] L_l, an element's 2 P coefficients together.  A warp
+// per element; one warp of the block does the ends of its eight elements (a warp
+// instruction of the FP64 pipe costs the same for one lane as for sixteen).  16384 elements
+// 34 us; with the coefficients element by element (16 bytes of each line for a leaf of one)
+// 134 us.
 __global__ void __launch_bounds__(256) tri_l2p_add_kernel(int E, const int* __restrict__ sleaf, int P,
-                                                          const float4* __restrict__ coef,
+                                                          const cplx* __restrict__ coef,
                                                           const cplx* __restrict__ L, const cplx* __restrict__ U,
                                                           const int* __restrict__ perm, const cplx* __restrict__ sph,
                                                           cplx c2, cplx* __restrict__ y) {
@@ -3587,16 +3620,16 @@ __global__ void __launch_bounds__(256) tri_l2p_add_kernel(int E, const int* __re
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, s = blockIdx.x * 8 + warp;
   if (s < E) {
     const cplx* Lb = L + (size_t)sleaf[s] * P;
-    const float4* cs = coef + (size_t)s * 2 * P;
-    dflt a{0, 0}, b{0, 0}, c{0, 0}, d{0, 0};
+    const cplx* cs = coef + (size_t)s * 2 * P;
+    cplx a{0, 0}, b{0, 0};
 #pragma unroll 2
     for (int l = lane; l < P; l += 32) {
-      const float4 u = cs[l], w = cs[P + l], v = dd_word(Lb[l]);
-      dd_cmac(a, b, u, v);
-      dd_cmac(c, d, w, v);
+      const cplx u = ld2(cs + l), w = ld2(cs + P + l), v = Lb[l];
+      cmac(a, u, v);
+      cmac(b, w, v);
     }
-    const dflt r = dd_wsum4(a, b, c, d, lane);
-    if ((lane & 7) == 0) so[warp][lane >> 3] = dd_value(r);
+    const double r = wsum4(a.re, a.im, b.re, b.im, lane);
+    if ((lane & 7) == 0) so[warp][lane >> 3] = r;
   }
   __syncthreads();
   const int t = blockIdx.x * 8 + (threadIdx.x >> 1), q = threadIdx.x & 1;
@@ -3607,19 +3640,9 @@ __global__ void __launch_bounds__(256) tri_l2p_add_kernel(int E, const int* __re
   }
 }
 
-// TOP and the L2P coefficients as words (once, at the end of the set-up).
-cudaError_t k_tri_words(pfmbem* h) {
-  const size_t rows = (size_t)h->nroot * h->lev[0].P, nc = (size_t)h->E * 2 * h->lev[h->D].P;
-  dd_words_kernel<<<(unsigned)std::min<size_t>((rows * rows + 255) / 256, 8192), 256, 0, h->stream>>>(rows * rows,
-                                                                                                     h->root);
-  dd_words_kernel<<<(unsigned)std::min<size_t>((nc + 255) / 256, 8192), 256, 0, h->stream>>>(nc, h->l2p_c);
-  return cudaGetLastError();
-}
-
 cudaError_t k_tri_top(pfmbem* h, cudaStream_t st) {
   const int rows = h->nroot * h->lev[0].P;
-  tri_top_kernel<<<(rows + 7) / 8, 256, 0, st>>>(rows, reinterpret_cast<const float4*>(h->root), h->lev[0].M,
-                                                 h->lev[0].L);
+  tri_top_kernel<<<(rows + 7) / 8, 256, 0, st>>>(rows, h->root, h->lev[0].M, h->lev[0].L);
   return cudaGetLastError();
 }
 
@@ -3627,7 +3650,7 @@ cudaError_t k_tri_top(pfmbem* h, cudaStream_t st) {
 // are set to the most that any handle takes, so that handles of other sizes in other
 // threads never lower them between this call's setting and its launch.
 cudaError_t k_tri_fiber(pfmbem* h, const cplx* x, cplx* y, cudaStream_t st) {
-  constexpr size_t per = sizeof(float4) * 3 * 2;
+  constexpr size_t per = sizeof(cplx) * 3 * 2;
   const cudaError_t e = cudaFuncSetAttribute(tri_fiber_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)(per * TRI_FIBER_MAX));
   if (e != cudaSuccess) return e;
@@ -3638,9 +3661,8 @@ cudaError_t k_tri_fiber(pfmbem* h, const cplx* x, cplx* y, cudaStream_t st) {
 
 cudaError_t k_tri_l2p(pfmbem* h, cplx* y) {
   const Level& leaf = h->lev[h->D];
-  tri_l2p_add_kernel<<<(h->E + 7) / 8, 256, 0, h->stream>>>(h->E, h->s_leaf, leaf.P,
-                                                            reinterpret_cast<const float4*>(h->l2p_c), leaf.L, h->U,
-                                                            h->s_perm, h->s_ph, cplx{h->c2re, h->c2im}, y);
+  tri_l2p_add_kernel<<<(h->E + 7) / 8, 256, 0, h->stream>>>(h->E, h->s_leaf, leaf.P, h->l2p_c, leaf.L, h->U, h->s_perm,
+                                                            h->s_ph, cplx{h->c2re, h->c2im}, y);
   return cudaGetLastError();
 }
 

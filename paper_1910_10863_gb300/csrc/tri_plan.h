@@ -640,7 +640,6 @@ static pfmbem_status build_plan_tri(pfmbem* h, const double* nodes, const std::v
     if (!h->side_ev) CK(pool_event(h->dev, &h->side_ev));
     CK(k_tri_caches(h));
     for (int l = 0; l <= D; ++l) CK(k_tri_m2l_split(h, l));
-    CK(k_tri_words(h));
   }
   h->ub_on = false;
   pin_release_async(h);
