@@ -985,7 +985,7 @@ __global__ void p2m_f64_kernel(const int* __restrict__ ne, const int* __restrict
                                const double2* __restrict__ sc, const double2* __restrict__ st,
                                const double2* __restrict__ snu, const double* __restrict__ sh,
                                const cplx* __restrict__ dens, cplx* __restrict__ Mout,
-                               const double2* __restrict__ ctr) {
+                               const double2* __restrict__ ctr, bool turn) {
   const int box = ne[blockIdx.x];
   const int P = 2 * p + 1;
   const size_t row = wgt ? box : blockIdx.x;      // no weights: unscaled, a row per listed box
@@ -1024,8 +1024,9 @@ __global__ void p2m_f64_kernel(const int* __restrict__ ne, const int* __restrict
     cplx a = (cw * 0.5 * k) * ph;
     cplx bcoef = (-eta * cw) * mul_i(va);
     cplx nuc{nu.x, nu.y};
-    // every thread begins at another coefficient: in step they would all add to one word
-    for (int i = 0, j = threadIdx.x % P; i < P; ++i, j = j + 1 < P ? j + 1 : 0) {
+    // turn: every thread begins at another coefficient, for in step they all add to one word
+    // (887 -> 346 us a launch on 16384 elements)
+    for (int i = 0, j = turn ? threadIdx.x % P : 0; i < P; ++i, j = j + 1 < P ? j + 1 : 0) {
       cplx v = a * (conj(nuc) * Jm[j] - nuc * Jm[j + 2]) + bcoef * Jm[j + 1];
       double iw = wgt ? 1.0 / wgt[j] : 1.0;
       atomicAdd(&acc[2 * j], v.re * iw);
@@ -2433,9 +2434,10 @@ cudaError_t k_build_fmm_caches(pfmbem* h) {
 // level 0); their local expansions come from the operator between the cells
 // (top_apply_kernel, in the product).
 // one_sum (the field u): the multipoles by the elements' integrals and M2M in one sum a
-// coefficient.  Where a density radiates almost nothing, the field from the far images
-// is what other terms of the size of 1 cancel to 1e-8, and the cached coefficients and
-// M2M in shares, each as accurate, moved u by 1e-9 to 6e-9 of itself.
+// coefficient, the threads of P2M in step.  Where a density radiates almost nothing, the
+// field from the far images is what other terms of the size of 1 cancel to 1e-8, and the
+// cached coefficients and M2M in shares, each as accurate, moved u by 1e-9 to 6e-9 of
+// itself; P2M's threads out of step by 0.4e-9 to 0.7e-9.
 static void upward_f64(pfmbem* h, const cplx* x, bool one_sum = false) {
   cudaStream_t st = h->stream;
   const int E = h->E, D = h->D;
@@ -2450,7 +2452,7 @@ static void upward_f64(pfmbem* h, const cplx* x, bool one_sum = false) {
   else
     p2m_f64_kernel<<<leaf.nne, 128, 0, st>>>(leaf.ne, leaf.box_begin, leaf.box_end, D, leaf.d, leaf.p, leaf.w_dev,
                                               h->g_far, h->k, h->eta, h->x0, h->y0, h->s_c, h->s_t, h->s_nu, h->s_h,
-                                              h->dens, leaf.M, leaf.ctr);
+                                              h->dens, leaf.M, leaf.ctr, !one_sum);
   prof_end(h, PH_P2M);
   for (int l = D - 1; l >= 0; --l) {
     Level& a = h->lev[l];
@@ -3296,7 +3298,7 @@ static void field_rules(pfmbem* h, FieldLeaf& fl, cplx* M, double2* hr) {
   for (int g = 2; g <= 4; ++g)
     p2m_f64_kernel<<<fl.nleaf, 128, 0, h->stream>>>(fl.ne, fl.bb, fl.be, h->D, L.d, L.p, nullptr, g, h->k, h->eta,
                                                     h->x0, h->y0, h->s_c, h->s_t, h->s_nu, h->s_h, h->dens,
-                                                    M + (size_t)(g - 2) * fl.nleaf * L.P, L.ctr);
+                                                    M + (size_t)(g - 2) * fl.nleaf * L.P, L.ctr, true);
   fl.M = M;
   fl.hr = hr;
 }
