@@ -2977,23 +2977,23 @@ __global__ void __launch_bounds__(128) field_direct_kernel(
 // H^+_{n+1}), and only the elements of the remaining leaves by quadrature.  A box
 // is far enough when its radius (half an element length added: elements stick out
 // of their box) is at most theta_l of its distance, theta_l = min(0.26,
-// 10^{-14.7/(p+1)}): the expansion's remainder falls like theta^(p+1), 2e-15 of
-// the box's field.  The field itself stays directly summed: where a density
-// radiates almost nothing, u cancels to 1e-6 of its terms, and the two forms'
-// remainders (1e-14 per element in the quadrature ladder) show at 2e-8 of it, the
-// derivative's at 1e-12.
+// 10^{-18/(p+1)}): the remainder of a monopole falls like theta^(p+1), that of a
+// dipole's derivative is (p + 1) / theta times as large, 2e-16 of the box's field
+// (at 10^{-14.7/(p+1)} it was 2e-13 at p = 20; a point costs a tenth more).
+// The field itself stays directly summed (field_direct_kernel).
 // One block per point walks the levels; the boxes that are too near are listed in
 // shared memory and their children tested at the next level.  FT_CAP holds every
 // list: the boxes of one level are disjoint and a listed one lies within (R + h/2)
-// / theta + R of the point, which at the smallest theta of the rule (0.1995 at
-// p = 20) and the longest element (a quarter of a leaf) is the area of 75 squares,
-// 128 triangles or 64 hexagonal cells.  The blocks from npts on evaluate the local
+// / theta + R of the point, which at the smallest theta of the rule (0.139 at
+// p = 20) and the longest element (a quarter of a leaf) is the area of 141 squares,
+// 242 triangles or 121 hexagonal cells (a box that found no room would be summed by
+// its elements at once).  The blocks from npts on evaluate the local
 // expansions, one point per thread.
 // FP64 arithmetic bounds it, about 0.5 million FP64 operations a point (some 300
 // expansions of 600 and the near elements); the direct sum has 3 E pairs of about
 // 400, 20 million on 16384 elements.  ETC with 256 points on 6144 elements: 25.5 ->
 // 0.93 ms.
-constexpr int FT_CAP = 160, FT_NT = 256;
+constexpr int FT_CAP = 256, FT_NT = 256;
 struct FieldTree {
   int D, nroot, nch0;
   int p[PF_MAXLEVEL + 1];
@@ -3042,6 +3042,23 @@ __device__ __forceinline__ cplx multipole_dx1(double k, double vx, double vy, in
   return (0.5 * k) * d;
 }
 
+// The x1-derivative at x of elements f0 .. f1 by quadrature, y moved by m periods.
+__device__ __noinline__ cplx elements_dx1(double2 x, int f0, int f1, double my, double k, double eta,
+                                          const double2* __restrict__ sc, const double2* __restrict__ st,
+                                          const double2* __restrict__ snu, const double* __restrict__ sh,
+                                          const cplx* __restrict__ dens) {
+  cplx d{0, 0};
+  for (int f = f0; f < f1; ++f) {
+    double2 c = sc[f];
+    c.y += my;
+    const double q = sqrt((x.x - c.x) * (x.x - c.x) + (x.y - c.y) * (x.y - c.y)) / sh[f];
+    cplx S{0, 0}, Dv{0, 0}, K{0, 0}, T{0, 0};
+    pair4_f64(k, x, double2{1.0, 0.0}, c, st[f], snu[f], sh[f], gl_order(q, 0), S, Dv, K, T);
+    d += T * dens[2 * f] - eta * mul_i(K * dens[2 * f + 1]);
+  }
+  return d;
+}
+
 __global__ void __launch_bounds__(FT_NT) field_tree_kernel(
     const __grid_constant__ FieldTree ft, int npts, const double2* __restrict__ pts, double k, double eta, double H,
     double ox, double oy, double x0, double y0, int mdir, cplx alpha, const double2* __restrict__ sc,
@@ -3085,6 +3102,9 @@ __global__ void __launch_bounds__(FT_NT) field_tree_kernel(
         if (o < FT_CAP) {
           s_box[cur][o] = box;
           s_img[cur][o] = m;
+        } else {
+          dacc += ipow_phase(alpha, m) *
+                  elements_dx1(x, ft.bb[l][box], ft.be[l][box], m * H, k, eta, sc, st, snu, sh, dens);
         }
       }
     }
@@ -3316,8 +3336,7 @@ static bool field_tree(const pfmbem* h, FieldTree& ft) {
     const Level& L = h->lev[l];
     const double R = (h->tree == 1 ? 0.5 : 0.5 * sqrt(2.0)) * L.d, kd = 2.0 * h->k * R;
     if (L.p < 20 || L.p < kd + 1.8 * pow(10.0, 2.0 / 3.0) * cbrt(kd)) return false;
-    const double theta = fmin(0.26, pow(10.0, -14.7 / (L.p + 1)));
-    const double far = (R + 0.5 * h->hmax) / theta;
+    const double far = (R + 0.5 * h->hmax) / fmin(0.26, pow(10.0, -18.0 / (L.p + 1)));
     ft.p[l] = L.p;
     ft.d[l] = L.d;
     ft.far2[l] = far * far;
