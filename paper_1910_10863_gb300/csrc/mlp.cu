@@ -397,9 +397,10 @@ bool is_dev(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Memory that the network's kernels may read and write in place: its own device's
-// (another device's is copied, as host memory is).
+// Memory that the network's kernels may read and write in place: its own device's, aligned
+// to its floats (another device's, or at an odd byte, is copied, as host memory is).
 bool is_local(const pfmbem_mlp* m, const void* p) {
+  if (reinterpret_cast<uintptr_t>(p) % alignof(float) != 0) return false;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
