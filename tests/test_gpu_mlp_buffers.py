@@ -71,3 +71,45 @@ def test_unaligned_device_buffers(pf):
     assert pf.lib().pfmbem_mlp_forward(net.h, BATCH, xp, yp) == 0
     assert train(pf, net, xp, tp, grad=gp) == 0
     assert torch.equal(back(yr).view_as(Y), Y) and torch.equal(back(gr), G)
+
+
+def test_step_with_a_device_gradient(pf):
+    """Adam reads the gradient where the pass wrote it, in the caller's buffer or the network's own: the same parameters
+    bit for bit after three steps."""
+    import torch
+    X, T = batch(1)
+    out = []
+    for where in ("device", "host", "none"):
+        net = pf.MLP(N_IN, HIDDEN, LAYERS, N_OUT, seed=5)
+        p = net.get_params()
+        g = {"device": torch.zeros(len(p), device="cuda"), "host": np.zeros(len(p), np.float32), "none": None}[where]
+        for _ in range(3):
+            assert train(pf, net, X, T, lr=1e-3, grad=g) == 0
+        q = net.get_params()
+        assert np.abs(q - p).max() > 1e-4
+        out.append(q)
+    assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+
+
+def test_buffers_that_share_memory(pf):
+    """An output over the input, and a gradient over the batch: as with buffers of their own."""
+    import torch
+    net = pf.MLP(N_IN, HIDDEN, LAYERS, N_OUT)
+    X, T = batch(2)
+    n = net.nparams()
+    Y, G = torch.zeros(BATCH, N_OUT, device="cuda"), torch.zeros(n, device="cuda")
+    assert pf.lib().pfmbem_mlp_forward(net.h, BATCH, pf.addr(X), pf.addr(Y)) == 0
+    assert train(pf, net, X, T, grad=G) == 0
+    for at in (0, 5, BATCH * N_IN - 1):                    # Y from X's first, fifth, last entry on
+        buf = torch.zeros(BATCH * (N_IN + N_OUT), device="cuda")
+        buf[:X.numel()] = X.flatten()
+        torch.cuda.synchronize()
+        assert pf.lib().pfmbem_mlp_forward(net.h, BATCH, buf.data_ptr(), buf.data_ptr() + 4 * at) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(buf[at:at + Y.numel()].view_as(Y), Y)
+    for first in (X, T):                                   # the gradient over X, then over T
+        buf = torch.zeros(max(n, first.numel()), device="cuda")
+        buf[:first.numel()] = first.flatten()
+        a = (buf, T) if first is X else (X, buf)
+        assert train(pf, net, a[0], a[1], grad=buf) == 0
+        assert torch.equal(buf[:n], G)
