@@ -26,11 +26,11 @@ struct pfmbem_mlp {
   float* m2 = nullptr;             // Adam second moment
   int64_t step = 0;
   int cap = 0;                     // batch capacity of the work buffers
-  std::vector<float*> act;         // activations per layer boundary [cap][dims[l]] (0: a host batch)
+  std::vector<float*> act;         // activations per layer boundary [cap][dims[l]] (0: a host batch; the last:
+                                   // the output, or a host batch's targets in training)
   std::vector<float*> pre;         // pre-activations per hidden layer
   float* dA = nullptr;             // work: gradient w.r.t. pre-activations, two in turn
   float* dB = nullptr;
-  float* tgt = nullptr;            // a host batch's targets
   float* loss = nullptr;           // device scalar
 };
 
@@ -62,8 +62,8 @@ struct Mat {
 };
 
 // Element e of a [TK][T] tile staged from an operand along k (KM) or across it: a
-// warp covers 8 k x 4 rows (32-byte sectors; with a row stride of 4 mod 32 or 20
-// words its stores meet 32 different banks), or rows one after another.
+// warp covers 8 k x 4 rows (32-byte sectors; with a row stride of 4 mod 32 words, 36 or
+// 68 here, its stores meet 32 different banks), or rows one after another.
 template <bool KM, int T>
 __device__ __forceinline__ void tile_at(int e, int& k, int& m) {
   if (KM) {
@@ -329,8 +329,7 @@ cudaError_t ensure_cap(pfmbem_mlp* m, int B) {
   for (float* p : m->pre) cudaFree(p);
   cudaFree(m->dA);
   cudaFree(m->dB);
-  cudaFree(m->tgt);
-  m->dA = m->dB = m->tgt = nullptr;
+  m->dA = m->dB = nullptr;
   m->cap = 0;
   m->act.assign(m->dims.size(), nullptr);
   m->pre.assign(m->dims.size(), nullptr);
@@ -342,7 +341,6 @@ cudaError_t ensure_cap(pfmbem_mlp* m, int B) {
   }
   if (cudaMalloc(&m->dA, sizeof(float) * (size_t)B * wmax) != cudaSuccess) return cudaErrorMemoryAllocation;
   if (cudaMalloc(&m->dB, sizeof(float) * (size_t)B * wmax) != cudaSuccess) return cudaErrorMemoryAllocation;
-  if (cudaMalloc(&m->tgt, sizeof(float) * (size_t)B * m->out) != cudaSuccess) return cudaErrorMemoryAllocation;
   m->cap = B;
   return cudaSuccess;
 }
@@ -613,7 +611,6 @@ void pfmbem_mlp_destroy(pfmbem_mlp_t m) {
   for (float* p : m->pre) cudaFree(p);
   cudaFree(m->dA);
   cudaFree(m->dB);
-  cudaFree(m->tgt);
   delete m;
 }
 
@@ -661,8 +658,9 @@ pfmbem_status pfmbem_mlp_train(pfmbem_mlp_t m, int B, const float* X, const floa
     X = m->act[0];
   }
   if (!is_local(m, T)) {
-    if (copy_in(m, m->tgt, T, (size_t)B * m->out) != cudaSuccess) return PFMBEM_ECUDA;
-    T = m->tgt;
+    // (a training pass leaves the output's place free: it writes the loss gradient to dA)
+    if (copy_in(m, m->act.back(), T, (size_t)B * m->out) != cudaSuccess) return PFMBEM_ECUDA;
+    T = m->act.back();
   }
   float* g = m->grad;
   if (grad && is_local(m, grad)) {
