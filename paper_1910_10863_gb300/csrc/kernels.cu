@@ -865,24 +865,23 @@ __device__ __forceinline__ void bessel01(double x, double& J0, double& J1, doubl
 // functions above, for the scattered field itself: where a density radiates almost
 // nothing u cancels to 1e-8 of its terms, and another rounding of these functions shows
 // at 1e-8 of u (the joint interpolants take half the time).  Per-term constants of the
-// series, m = 1..39: 1/m^2, 1/(m(m+1)), H_m and 2 H_m + 1/(m+1) - 2 gamma.
-__constant__ double c_ser_im2[40], c_ser_imm1[40], c_ser_H[40], c_ser_y1[40];
+// series, m = 1..39: 1/m^2, 1/(m(m+1)), H_m and 2 H_m + 1/(m+1) - 2 gamma, a term's four
+// together: as four arrays beside the interpolants' tables they cost field maps of few
+// points 3 to 5 % (one warp an SM sub-partition, and its constant loads in the chain).
+struct alignas(16) SerTerm {
+  double im2, imm1, H, y1;
+};
+__constant__ SerTerm c_ser[40];
 
 void k_upload_series() {
-  double im2[40] = {0}, imm1[40] = {0}, H[40] = {0}, y1c[40] = {0};
+  SerTerm t[40] = {};
   const double EG = 0.57721566490153286061;
   double Hm = 0.0;
   for (int m = 1; m < 40; ++m) {
-    im2[m] = 1.0 / ((double)m * m);
-    imm1[m] = 1.0 / ((double)m * (m + 1));
     Hm += 1.0 / m;
-    H[m] = Hm;
-    y1c[m] = 2.0 * Hm + 1.0 / (m + 1) - 2.0 * EG;
+    t[m] = SerTerm{1.0 / ((double)m * m), 1.0 / ((double)m * (m + 1)), Hm, 2.0 * Hm + 1.0 / (m + 1) - 2.0 * EG};
   }
-  cudaMemcpyToSymbol(c_ser_im2, im2, sizeof(im2));
-  cudaMemcpyToSymbol(c_ser_imm1, imm1, sizeof(imm1));
-  cudaMemcpyToSymbol(c_ser_H, H, sizeof(H));
-  cudaMemcpyToSymbol(c_ser_y1, y1c, sizeof(y1c));
+  cudaMemcpyToSymbol(c_ser, t, sizeof(t));
 }
 
 __device__ __forceinline__ void bessel01_series(double x, double& J0, double& J1, double& Y0, double& Y1) {
@@ -900,12 +899,13 @@ __device__ __forceinline__ void bessel01_series(double x, double& J0, double& J1
   const int mmax = x < 0.5 ? 10 : (x < 1.5 ? 15 : (x < 3.0 ? 21 : 27));
 #pragma unroll 1
   for (int m = 1; m < mmax; ++m) {
-    a *= -h2 * c_ser_im2[m];
-    b *= -h2 * c_ser_imm1[m];
+    const SerTerm t = c_ser[m];
+    a *= -h2 * t.im2;
+    b *= -h2 * t.imm1;
     sJ0 += a;
     sJ1 += b;
-    sY0 = fma(-c_ser_H[m], a, sY0);           // (-1)^{m+1} H_m (x/2)^{2m}/(m!)^2
-    sY1 = fma(-c_ser_y1[m], b, sY1);
+    sY0 = fma(-t.H, a, sY0);           // (-1)^{m+1} H_m (x/2)^{2m}/(m!)^2
+    sY1 = fma(-t.y1, b, sY1);
   }
   const double L = log(h);
   J0 = sJ0;
@@ -2921,7 +2921,9 @@ __global__ void field_finish_kernel(int npts, const double2* __restrict__ pts, i
 // (k/2) sum_m J_m(kr) e^{i m theta} (c_{m+1} - c_{m-1}).
 // With a row of roots the direct images are |m| <= mdir = m0 - 1 and the local
 // expansion is the super root's (centre (ox, oy)); one root: mdir = 1, the root's.
-// One warp per (point, slice): slice q of nsl takes every nsl-th group of 32 of
+// One warp and block per (point, slice), so that few points spread over the SMs and many
+// even out (634 points on 3350 elements 28.7 -> 19.2 ms, 11 points on 1296 4.47 -> 4.11
+// against blocks of four): slice q of nsl takes every nsl-th group of 32 of
 // the (element, image) pairs and leaves its sums in part[point][q]; the local
 // expansions are separate threads (the last blocks) and go to part[point][nsl];
 // field_finish_kernel adds a point's parts in order.  Bound by the FP64 pipe.  The
@@ -2931,18 +2933,16 @@ __global__ void field_finish_kernel(int npts, const double2* __restrict__ pts, i
 // shows at 2e-9 to 7e-9 of u (1024 points on 16384 elements: 117 ms; 74 ms with the
 // joint interpolants, 64 ms with slices too).
 template <bool WU, bool WD>
-__global__ void __launch_bounds__(128) field_direct_kernel(
+__global__ void __launch_bounds__(32) field_direct_kernel(
     int npts, const double2* __restrict__ pts, int nsl, int E, double k, double eta, double H, double ox, double oy,
     double y0, int mdir, cplx alpha, const double2* __restrict__ sc, const double2* __restrict__ st,
     const double2* __restrict__ snu, const double* __restrict__ sh, const cplx* __restrict__ dens, int p0,
     const double* __restrict__ w0, const cplx* __restrict__ L0, cplx* __restrict__ part) {
-  const int nb = (int)(((int64_t)npts * nsl + 3) >> 2);       // blocks of the sums
-  if ((int)blockIdx.x >= nb) {
-    local_part(((int)blockIdx.x - nb) * 128 + threadIdx.x, npts, pts, nsl, k, H, ox, oy, y0, p0, w0, L0, part);
+  const int lane = threadIdx.x, w = blockIdx.x;
+  if (w >= npts * nsl) {
+    local_part((w - npts * nsl) * 32 + lane, npts, pts, nsl, k, H, ox, oy, y0, p0, w0, L0, part);
     return;
   }
-  const int lane = threadIdx.x & 31, w = blockIdx.x * 4 + (threadIdx.x >> 5);
-  if (w >= npts * nsl) return;
   const int pi = w / nsl, sl = w - pi * nsl;
   double2 x = pts[pi];
   x.y -= floor((x.y - y0) / H) * H;
@@ -3407,9 +3407,9 @@ cudaError_t k_field(pfmbem* h, int npts, const double2* pts, cplx* u, cplx* dudx
         fl, npts, pts, nsl, h->k, h->eta, h->H, ox, oy, h->x0, h->y0, mdir, h->alpha, h->s_c, h->s_t, h->s_nu, h->s_h,
         h->dens, p0, w0, L0, part);
   } else {
-    const unsigned grid = (unsigned)(((int64_t)npts * nsl + 3) / 4 + (npts + 127) / 128);
+    const unsigned grid = (unsigned)((int64_t)npts * nsl + (npts + 31) / 32);
     auto launch = [&](auto kern) {
-      kern<<<grid, 128, 0, h->stream>>>(npts, pts, nsl, h->E, h->k, h->eta, h->H, ox, oy, h->y0, mdir, h->alpha,
+      kern<<<grid, 32, 0, h->stream>>>(npts, pts, nsl, h->E, h->k, h->eta, h->H, ox, oy, h->y0, mdir, h->alpha,
                                         h->s_c, h->s_t, h->s_nu, h->s_h, h->dens, p0, w0, L0, part);
     };
     if (u && dudx1) launch(field_direct_kernel<true, true>);
