@@ -490,6 +490,8 @@ cudaError_t batch_fill(pfmbem* h, int GS, FusedArgs<C>& a) {
   }
   {
     const int nf = h->fz_nfft + h->fz_nchunk;
+    // (the FP64 products of a batch are few: their P2M's larger weight, as in launch_fused,
+    // changes 2 to 32 instances by less than 1 %)
     const double wa = (double)h->lev[h->D].nne / FW;
     const int fb = (int)((double)GS * nf / (nf + wa) + 0.5);
     a.fblk = GS >= 16 ? std::max(1, std::min({fb, nf, GS - GS / 4})) : 0;

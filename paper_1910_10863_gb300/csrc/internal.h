@@ -454,6 +454,7 @@ cudaError_t k_tri_caches(pfmbem* h);
 cudaError_t k_tri_m2l_split(pfmbem* h, int l);
 cudaError_t k_tri_m2l_dd(pfmbem* h);
 size_t k_tri_m2l_smem(int P);
+constexpr int PF_SMS = 152;                   // SMs of a GB300, for splits of the work alone
 constexpr int TRI_FIBER_MAX = 1024;           // most elements of a fiber with cached tables
 constexpr size_t TRI_M2L_SMEM = 200 * 1024;   // above it a level's M2L goes target by target
 cudaError_t k_tri_top(pfmbem* h, cudaStream_t st);

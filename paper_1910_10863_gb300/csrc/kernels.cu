@@ -761,9 +761,8 @@ extern "C" pfmbem_status pfmbem_lattice_sums_noalloc(double k, double H, double 
 // instruction per 16 cycles and SM), so the number of FP64 instructions is their
 // time: about 100 in each range.  The forms before took up to 27 terms of six
 // (series, x <= 4) or CUDA's four functions, each with its own amplitude, phase
-// and sine.  A create of the 24-fiber round-square crystal (512 x 512 blocks) takes
-// 7.2 instead of 9.6 ms, a field map of 1024 points on 16384 elements 74 instead of
-// 118 ms (directly summed).
+// and sine.  A create of the 24-fiber round-square crystal (512 x 512 blocks) took
+// 7.2 instead of 9.6 ms with them.
 __constant__ double c_bes_lo[4][15] = {
     {1.0, -0.25, 0.015625, -0.00043402777777777775, 6.781684027777777e-06, -6.781684027777778e-08,
      4.709502797067901e-10, -2.4028075495244395e-12, 9.385966990329842e-15, -2.896903392077112e-17,
@@ -1783,7 +1782,7 @@ __global__ void near_sources_kernel(const int* __restrict__ nl_ptr, const int* _
 static void fiber_build_plane(pfmbem* h, bool ktab, cudaStream_t st) {
   cplx c2{h->c2re, h->c2im};
   prof_begin(h, PH_BUILD);
-  const int sp = (int64_t)h->nfb_rows * h->max_fiber >= 152 * 2048 ? 1 : 4;   // pairs for every resident thread
+  const int sp = (int64_t)h->nfb_rows * h->max_fiber >= PF_SMS * 2048 ? 1 : 4;   // pairs for every resident thread
   auto kern = sp == 1 ? fiber_build_kernel<1> : fiber_build_kernel<4>;
   kern<<<dim3(h->nfb_rows, (h->max_fiber + 128 / sp - 1) / (128 / sp), 1), 128, 0, st>>>(
       h->fb_rows, h->o_fiber, h->fib_off, h->fb_base, h->k, h->k1, h->eta, h->rho, c2, h->o_c, h->o_t, h->o_nu,
@@ -3380,7 +3379,7 @@ cudaError_t k_field(pfmbem* h, int npts, const double2* pts, cplx* u, cplx* dudx
   auto slices = [&]() -> int {
     if (tree || u) return 1;      // u: one order of its sum (field_direct_kernel)
     const int64_t terms = (int64_t)(2 * mdir + 1) * (leaf ? fl.nleaf : h->E);
-    return (int)std::max<int64_t>(1, std::min<int64_t>((152 * (leaf ? 8 : 32) + npts - 1) / npts, terms / 256));
+    return (int)std::max<int64_t>(1, std::min<int64_t>((PF_SMS * (leaf ? 8 : 32) + npts - 1) / npts, terms / 256));
   };
   int nsl = slices();
   void* buf = nullptr;

@@ -7,21 +7,23 @@
 // separates them with a device-wide barrier:
 //
 //   A   gather the densities into tree order (alpha^{-m0} phase), P2M and
-//       clear the local expansions of levels 1..D (warp per leaf); at the
+//       clear the local expansions of levels 1..D (warp per leaf; in the FP64
+//       product per leaf and 32 coefficients); at the
 //       same time a share of the blocks applies the same-fiber blocks of
 //       eq. 9 to x and writes them to y: a regular-polygon fiber whose
 //       element count is a power of two by FFT (block per fiber), the others
 //       by cached rows (block per chunk of 32 rows)
-//   B_l M2M into level l = D-1 .. 0 (warp per box, or per output coefficient
-//       where the boxes are few); the root stage forms L(0) directly from the
+//   B_l M2M into level l = D-1 .. 0 (warp per box, block per box in the FP64
+//       product, or warp per output coefficient where the boxes are few); the root stage forms L(0) directly from the
 //       four level-1 multipoles through the folded operator R T_0.  The
 //       cached near-field sums of all elements are spread evenly over these
 //       stages, whose few boxes leave most warps idle        (warp per element)
-//   D_l L2L from the parent (warp per box or per coefficient) and M2L (warp
-//       per pair, or block per chunk of pairs with one translation offset and
-//       T_o staged in shared memory), both added atomically into L(l)
+//   D_l L2L from the parent (warp per box or per coefficient) and M2L (block
+//       per chunk of pairs with one translation offset and T_o staged in shared
+//       memory; in the FP64 product, where a level's pairs are few, warp per
+//       pair, 32 targets and share of the sources), both added atomically into L(l)
 //   E   L2P plus the near-field sums, and the combination of eq. 9 added to
-//       the fiber part already in y                           (warp per element)
+//       the fiber part already in y   (warp per 32 elements, FP64 product per 16)
 //
 // Warp-level items are dealt round-robin over the blocks (item i to block
 // i mod grid), so that a stage with few items still spreads over all SMs: on
@@ -1901,7 +1903,9 @@ __device__ __forceinline__ void prefetch_l2p(const FusedArgs<C>& a, int bid, int
 }
 
 // The near-field blocks of the warp items of stage j of nst, about their share of the
-// array (rows are dealt by number, not by bytes), where that is no more than 16 MB.
+// array (rows are dealt by number, not by bytes), where that is no more than 16 MB: never,
+// up to 16 MB, always take 321, 293, 293 us on the 8x8 hexagon block, 320, 271, 294 on the
+// 16x16 square (64 elements a fiber), 1587, 1389, 1488 on the 32x32 square.
 template <class C>
 __device__ __forceinline__ void prefetch_near(const FusedArgs<C>& a, int j, int nst, int bid, int G) {
   const size_t n = (size_t)a.near_blocks * 4 * sizeof(cplxf), o0 = n / nst * j & ~(size_t)127;
@@ -1917,7 +1921,9 @@ __device__ __forceinline__ void prefetch_near(const FusedArgs<C>& a, int j, int 
 // the G blocks: the blocks with one block item less, if that ends sooner than all of
 // them (in units of a warp item, a block item takes R).  A block that carries an
 // operator's copy and its boxes then goes straight to the barrier instead of on to
-// near-field rows, which used to make it the stage's last.
+// near-field rows, which used to make it the stage's last.  R = 1, 3, 6 in the FP64
+// product: 8x8 hexagon 300, 293, 295 us, 32x32 square 1404, 1389, 1433; R = 1 or 2 in the
+// FP32 product within 4 % of each other.
 template <class C>
 __device__ __forceinline__ void warp_share(int N, int W, int rank, int warp, int G, int& wf, int& ws) {
   constexpr int R = sizeof(C) == sizeof(cplx) ? 3 : 1;
@@ -3128,7 +3134,9 @@ cudaError_t launch_fused(pfmbem* h, const cplx* x, cplx* y, bool f32, const int*
   {
     const int nf = h->fz_nfft + h->fz_nchunk;
     // (the FP64 product's P2M, two double-float warps a leaf, weighs 2.65 times as much:
-    // on the 32x32 block 304 fiber blocks were done in 63 us, the other 152 in 180)
+    // on the 32x32 block 304 fiber blocks were done in 63 us, the other 152 in 180.  The
+    // product at weights 1, 2.65, 4: 1467, 1389, 1400 us there, 293, 293, 305 us on the 8x8
+    // hexagon block)
     const double wa = (f32 ? 1.0 : 2.65) * (double)h->lev[h->D].nne / nwarp;
     const int fb = (int)((double)grid * nf / (nf + wa) + 0.5);
     a.fblk = grid >= 16 ? std::max(1, std::min({fb, nf, grid - grid / 4})) : 0;
@@ -3338,7 +3346,7 @@ __global__ void split_hl_kernel(size_t n, const cplx* __restrict__ a, cplxf* __r
 // read serves both and four sums are in flight, splits their phased source
 // multipoles alpha^m M(src), sums each target coefficient with error-free products
 // and sums (about 48 bits) and adds it to L(tgt) in FP64.  FP32 instructions bound
-// it: 65 384 pairs at P = 61 are 10 GFP32 instructions a lane.
+// it: 65 384 pairs at P = 61, 61^2 x 40 instructions each, are 9.7 G lane instructions.
 template <int NP>
 __device__ __forceinline__ void tri_m2l_pairs(int P, int pi, const int* __restrict__ ptgt, const int* __restrict__ psrc,
                                               const int* __restrict__ pimg, const float4* T, float4* wsm,
@@ -3688,7 +3696,7 @@ cudaError_t k_tri_m2m_dd(pfmbem* h, int l) {
   // time: 64 to 500 boxes 18 to 28 us, by 4 shares 32 us); 1139 boxes take 51 us by 16
   // and 34 us by 4, for the shares' ends then fill the chip
   const int nch = l == 0 ? 6 : 4;
-  const dim3 nt = tri_block(a.P, a.nne <= 4 * 152 ? TRI_Y : 4);
+  const dim3 nt = tri_block(a.P, a.nne <= 4 * PF_SMS ? TRI_Y : 4);
   const size_t smem = sizeof(float4) * std::max((size_t)nch * c.P, (size_t)nt.y * a.P);
   tri_m2m_dd_kernel<<<a.nne, nt, smem, h->stream>>>(a.ne, a.P, c.P, a.tri_nop, a.tri_m2m_hl, c.box_begin, c.box_end,
                                                     c.M, a.M, nch, c.pidx, a.L);
