@@ -602,7 +602,7 @@ cudaError_t k_batch_solve(int ninst, pfmbem* const* hs, const int* order, int GS
     // fewer instances than such groups, up to the blocks that the largest product on
     // the whole grid has work for.
     int need = 1;
-    for (int i = 0; i < ninst; ++i) need = std::max(need, hs[i]->fz_grid32);
+    for (int i = 0; i < ninst; ++i) need = std::max(need, hs[i]->fz_all32);
     GS = std::max(BATCH_GROUP, std::min(resident / ninst, need));
   }
   // groups large enough for the root's coefficients, one warp each

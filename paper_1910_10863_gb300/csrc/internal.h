@@ -267,7 +267,7 @@ struct pfmbem {
   cplxf* Uf = nullptr;           // [E][2]
   // single-launch cached matvec (cooperative grid, device-wide barrier)
   bool fused = false;
-  int fz_grid64 = 0, fz_grid32 = 0;
+  int fz_grid64 = 0, fz_grid32 = 0, fz_all32 = 0;   // all32: blocks that the FP32 product has work for
   int arn_grid = 0;              // blocks of the device-side GMRES step (0: host-side steps)
   unsigned long long* arn_bar = nullptr;   // its barrier's arrival counter
   unsigned long long* fz_bar = nullptr;    // [2] barrier arrival counters (FP64, FP32 product)

@@ -3794,11 +3794,21 @@ cudaError_t k_fused_prepare(pfmbem* h, bool* ok) {
   // leaves and over fibers or fiber row chunks (fiber part of A)
   int need = std::max(h->lev[h->D].nne, h->fz_nchunk + h->fz_nfft);
   for (int l = 0; l <= h->D; ++l) need = std::max(need, (h->lev[l].nne + FW - 1) / FW);
-  // and the near-field rows (a warp each) and M2L chunks (a block each): a small
-  // block's product is a chain of latencies, shorter over more SMs
-  need = std::max(need, (h->E + FW - 1) / FW);
-  for (int l = 1; l <= h->D; ++l) need = std::max(need, h->lev[l].nchunk);
   need = std::max(need, 1);
+  // and the near-field rows (a warp each) and M2L chunks (a block each): a small
+  // block's product is a chain of latencies, shorter over more SMs.  But products of
+  // several handles (threads, streams) run side by side only while their grids fit the
+  // chip together, so the further blocks leave room for as many products as fitted without
+  // them, up to three.  5x5 square of 80 elements a fiber, FP64, one product and four at
+  // a time: 166 and 79 us a product without them, 96 and 113 with all, 98 and 56 so; the sweep's
+  // blocks (2350 elements), FP32: 104 and 53, 80 and 78, 90 and 47; 4x4 square of 64, FP32:
+  // 131 and 36, 55 and 27, 55 and 20.
+  int more = (h->E + FW - 1) / FW;
+  for (int l = 1; l <= h->D; ++l) more = std::max(more, h->lev[l].nchunk);
+  auto blocks = [&](int resident, int beside) {
+    const int side = std::max(1, std::min(beside, resident / need));
+    return std::min(resident, std::max(need, std::min(more, resident / side)));
+  };
   // staging region of the FP32 product: room for the four stacked quadrant
   // operators of M2M and L2L at the FP32 orders, within about 100 KB per block
   // (two resident blocks per SM)
@@ -3832,10 +3842,11 @@ cudaError_t k_fused_prepare(pfmbem* h, bool* ok) {
     if (L.tc_fused && L.tc_Bf && L.tc_ntile > 0 && tc::kpad(fused_P(h, l, true)) <= TC_KPMAX)
       h->fz_tcb32 = std::max(h->fz_tcb32, tc_smem_bytes(tc::kpad(fused_P(h, l, true))));
   }
-  h->fz_grid64 = std::min(fused_grid<cplx, false>(h->max_fiber, TSIZE, 0), need);
-  h->fz_grid32 = std::min(h->fz_tcb32 > 0 ? fused_grid<cplxf, true>(h->max_fiber, h->fz_treg32, h->fz_tcb32)
-                                          : fused_grid<cplxf, false>(h->max_fiber, h->fz_treg32 + h->fz_tregL32, 0),
-                          need);
+  h->fz_grid64 = blocks(fused_grid<cplx, false>(h->max_fiber, TSIZE, 0), 3);
+  const int res32 = h->fz_tcb32 > 0 ? fused_grid<cplxf, true>(h->max_fiber, h->fz_treg32, h->fz_tcb32)
+                                    : fused_grid<cplxf, false>(h->max_fiber, h->fz_treg32 + h->fz_tregL32, 0);
+  h->fz_grid32 = blocks(res32, 3);
+  h->fz_all32 = blocks(res32, 1);
   {
     // PFMBEM_FUSED_GRID caps both grids (a test of the products on few blocks,
     // the group sizes of the batched launch; the cap is kept a multiple of 1)
@@ -3843,6 +3854,7 @@ cudaError_t k_fused_prepare(pfmbem* h, bool* ok) {
     if (fg && std::atoi(fg) > 0) {
       h->fz_grid64 = std::min(h->fz_grid64, std::atoi(fg));
       h->fz_grid32 = std::min(h->fz_grid32, std::atoi(fg));
+      h->fz_all32 = std::min(h->fz_all32, std::atoi(fg));
     }
   }
   if (h->fz_grid64 <= 0 || h->fz_grid32 <= 0) return cudaSuccess;
