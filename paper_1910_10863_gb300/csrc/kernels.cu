@@ -2929,8 +2929,8 @@ __global__ void field_finish_kernel(int npts, const double2* __restrict__ pts, i
 // derivative alone takes slices, for one warp per point leaves most of the chip idle
 // below some thousand points.  u takes one slice and the series' Bessel functions: its
 // terms are of the size of 1 where it may be 1e-8, so that another order of the sum
-// shows at 2e-9 to 7e-9 of u (1024 points on 16384 elements: 117 ms; 74 ms with the
-// joint interpolants, 64 ms with slices too).
+// shows at 2e-9 to 7e-9 of u (1024 points on 16384 elements: 104 ms; in blocks of four
+// warps 117 ms, with the joint interpolants 74 ms, with slices too 64 ms).
 template <bool WU, bool WD>
 __global__ void __launch_bounds__(32) field_direct_kernel(
     int npts, const double2* __restrict__ pts, int nsl, int E, double k, double eta, double H, double ox, double oy,
